@@ -1637,190 +1637,121 @@ __global__ void __launch_bounds__(256) kb_finalise_share(MemberTable t) {
 
 
 // ------------------------------------------------------------ normals
+// multiply-add with a weight that is a power of two: the product is exact, so
+// this is the same rounding as a separate multiply and add
+__device__ __forceinline__ float fma_pow2(float w, float d, float s) { return __fmaf_rn(w, d, s); }
+__device__ __forceinline__ double fma_pow2(double w, double d, double s) { return __fma_rn(w, d, s); }
+
 // Parker-Youngs gradient of phi at cell (x, y, z): per axis a, the centred
 // difference across the 3x3 block perpendicular to a with weights 4 (centre),
 // 2 (edges), 1 (corners), divided by 32; exact for linear phi.  An axis whose
 // block touches a wall or obstacle uses a two-point difference over the
 // non-obstacle cells instead (narrowed stencil near obstacles).  RC is the
 // compute type: FP64 in the FP64 path, FP32 otherwise.
+// The 27 values are loaded once each, all in flight together (the cell itself
+// stands in beyond a wall), and the flag bytes only where the domain holds
+// obstacle cells: a bit mask of the 27 cells decides each axis.
 template <class RC, class PT>
-__device__ inline void normal_py(const Geom& g, const uint8_t* flags, const PT* phi, int x,
-                                 int y, int z, RC* n) {
-  const int p[3] = {x, y, z};
-  const int c = x + g.sx * (y + g.ny * z);
+__device__ __forceinline__ void normal_py(const Geom& g, const uint8_t* flags, const PT* phi, int x,
+                                          int y, int z, RC* n) {
+  Nbr nb;
+  nb.setup(g, x, y, z);
+  const int c = nb.in(0, 0, 0);
+  RC v[27];
+  unsigned solid = 0;  // bit 9 (dz+1) + 3 (dy+1) + (dx+1): wall or obstacle
+#pragma unroll
+  for (int k = 0; k < 27; ++k) {
+    const int m = nb.at(k % 3 - 1, (k / 3) % 3 - 1, k / 9 - 1);
+    const int ms = m >= 0 ? m : c;
+    v[k] = (RC)phi[ms];
+    if (m < 0) solid |= 1u << k;
+    if (g.has_obst && (flags[ms] & F_TYPE) == T_OBST) solid |= 1u << k;
+  }
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
-    int b = (a + 1) % 3, cc = (a + 2) % 3;
-    if (b > cc) { int t = b; b = cc; cc = t; }
-    int yp_[9], ym_[9];
-    bool touches = false;
+    constexpr int st[3] = {1, 3, 9};
+    const int sa = st[a], sb = a == 0 ? 3 : 1, sc = a == 2 ? 3 : 9;
+    unsigned block = 0;  // the 18 cells of the two 3x3 blocks
+#pragma unroll
     for (int ob = -1; ob <= 1; ++ob)
-      for (int oc = -1; oc <= 1; ++oc) {
-        int dp[3] = {0, 0, 0}, dm[3] = {0, 0, 0};
-        dp[a] = 1; dm[a] = -1;
-        dp[b] += ob; dm[b] += ob;
-        dp[cc] += oc; dm[cc] += oc;
-        const int k = 3 * (ob + 1) + (oc + 1);
-        yp_[k] = nb_at(g, p[0], p[1], p[2], dp[0], dp[1], dp[2]);
-        ym_[k] = nb_at(g, p[0], p[1], p[2], dm[0], dm[1], dm[2]);
-        if (type_at(flags, yp_[k]) == T_OBST || type_at(flags, ym_[k]) == T_OBST) touches = true;
-      }
-    if (!touches) {
+#pragma unroll
+      for (int oc = -1; oc <= 1; ++oc)
+        block |= (1u << (13 + sa + ob * sb + oc * sc)) | (1u << (13 - sa + ob * sb + oc * sc));
+    if (!(solid & block)) {
       RC sum = (RC)0;
+#pragma unroll
       for (int ob = -1; ob <= 1; ++ob)
+#pragma unroll
         for (int oc = -1; oc <= 1; ++oc) {
-          const int k = 3 * (ob + 1) + (oc + 1);
           const RC w = (RC)((ob == 0 ? 2.0 : 1.0) * (oc == 0 ? 2.0 : 1.0));
-          const RC t = w * ((RC)phi[yp_[k]] - (RC)phi[ym_[k]]);
-          sum = (k == 0) ? (RC)0 + t : sum + t;
+          const int k = 13 + ob * sb + oc * sc;
+          sum = fma_pow2(w, v[k + sa] - v[k - sa], sum);
         }
       n[a] = sum / (RC)32;
     } else {
-      const int yp = yp_[4], ym = ym_[4];
-      const bool okp = type_at(flags, yp) != T_OBST, okm = type_at(flags, ym) != T_OBST;
-      if (okp && okm) n[a] = (RC)0.5 * ((RC)phi[yp] - (RC)phi[ym]);
-      else if (okp) n[a] = (RC)phi[yp] - (RC)phi[c];
-      else if (okm) n[a] = (RC)phi[c] - (RC)phi[ym];
+      const bool okp = !((solid >> (13 + sa)) & 1u), okm = !((solid >> (13 - sa)) & 1u);
+      if (okp && okm) n[a] = (RC)0.5 * (v[13 + sa] - v[13 - sa]);
+      else if (okp) n[a] = v[13 + sa] - v[13];
+      else if (okm) n[a] = v[13] - v[13 - sa];
       else n[a] = (RC)0;
     }
   }
 }
 
 template <class RC, class PT>
-__device__ inline void unit_normal(const Geom& g, const uint8_t* flags, const PT* phi, int x,
-                                   int y, int z, RC* nh) {
+__device__ __forceinline__ void unit_normal(const Geom& g, const uint8_t* flags, const PT* phi,
+                                            int x, int y, int z, RC* nh) {
   RC n[3];
   normal_py<RC>(g, flags, phi, x, y, z, n);
   const RC len = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-  if (len < (RC)1e-12) {
-    nh[0] = nh[1] = nh[2] = (RC)0;
-  } else {
-    nh[0] = n[0] / len;
-    nh[1] = n[1] / len;
-    nh[2] = n[2] / len;
-  }
+  const bool tiny = len < (RC)1e-12;
+  const RC l = tiny ? (RC)1 : len;
+  nh[0] = tiny ? (RC)0 : n[0] / l;
+  nh[1] = tiny ? (RC)0 : n[1] / l;
+  nh[2] = tiny ? (RC)0 : n[2] / l;
 }
 
-// coordinate v wrapped into [0, n) (periodic axes; v within one period)
-__device__ __forceinline__ int wrapc(int v, int n) {
-  if (v < 0) v += n;
-  else if (v >= n) v -= n;
-  return (v < 0 || v >= n) ? ((v % n) + n) % n : v;
-}
-
-// K = -div(n_hat), central differences over the face neighbours; a wall side
-// is replaced by the centre value.
+// K = -div(n_hat) of the cell c of each group of eight consecutive lanes
+// (c < 0: none), central differences over the face neighbours; a wall or
+// obstacle side is replaced by the centre value.  Lane 2a (2a + 1) of a group
+// forms the unit normal at the face neighbour c + e_a (c - e_a), lane 6 the
+// one at c itself where a side needs it; the group's lane 0 returns K.
+// Warp-uniform call.
+// Why eight lanes: one thread per cell ran six or seven 27-point stencils one
+// after another, through 50 KB of straight-line code, and near walls with a
+// flag test before every load, so that short lists waited for one thread's
+// chain (400 interface cells of a 750x200 FP64 dam break: 184 us) and long
+// lists for the few threads that take the wall path (40,000 cells of a Taylor
+// bubble in a tube, FP32: 176 us).
 template <class RC, class PT>
-__device__ inline RC curvature(const Geom& g, const uint8_t* flags, const PT* phi, int x,
-                               int y, int z) {
-  RC nc[3];
-  unit_normal<RC>(g, flags, phi, x, y, z, nc);
-  RC div = (RC)0;
-  for (int a = 0; a < 3; ++a) {
-    int dp[3] = {0, 0, 0}, dm[3] = {0, 0, 0};
-    dp[a] = 1; dm[a] = -1;
-    const int yp = nb_at(g, x, y, z, dp[0], dp[1], dp[2]);
-    const int ym = nb_at(g, x, y, z, dm[0], dm[1], dm[2]);
-    const bool okp = type_at(flags, yp) != T_OBST, okm = type_at(flags, ym) != T_OBST;
-    RC np[3], nm[3], dd;
-    const int px = wrapc(x + dp[0], g.nx), py = wrapc(y + dp[1], g.ny), pz = wrapc(z + dp[2], g.nz);
-    const int mx = wrapc(x + dm[0], g.nx), my = wrapc(y + dm[1], g.ny), mz = wrapc(z + dm[2], g.nz);
-    if (okp && okm) {
-      unit_normal<RC>(g, flags, phi, px, py, pz, np);
-      unit_normal<RC>(g, flags, phi, mx, my, mz, nm);
-      dd = (RC)0.5 * (np[a] - nm[a]);
-    } else if (okp) {
-      unit_normal<RC>(g, flags, phi, px, py, pz, np);
-      dd = np[a] - nc[a];
-    } else if (okm) {
-      unit_normal<RC>(g, flags, phi, mx, my, mz, nm);
-      dd = nc[a] - nm[a];
-    } else {
-      dd = (RC)0;
-    }
-    div = (a == 0) ? (RC)0 + dd : div + dd;
+__device__ __forceinline__ RC curvature8(const Geom& g, const uint8_t* flags, const PT* phi, int c) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, sub = lane & 7, base = lane & 24;
+  int px = 0, py = 0, pz = 0;
+  bool ok = false;
+  if (c >= 0 && sub < 7) {
+    int x, y, z;
+    cell_xyz(g, c, x, y, z);
+    const int s = (sub & 1) ? -1 : 1, a = sub >> 1;  // a = 3: the cell itself
+    const int n = nb_at(g, x, y, z, a == 0 ? s : 0, a == 1 ? s : 0, a == 2 ? s : 0);
+    ok = n >= 0 && (!g.has_obst || (flags[n] & F_TYPE) != T_OBST);
+    if (ok) cell_xyz(g, n, px, py, pz);
   }
-  return -div;
-}
-
-// The same curvature for a cell whose distance-2 neighbourhood holds no wall
-// or obstacle: no type checks, wrapped coordinates computed once.  Same
-// operation order as curvature(), so the results are identical.
-template <class RC, class PT>
-__device__ inline RC curvature_open(const Geom& g, const PT* phi, int x, int y, int z) {
-  int X[5], Y[5], Z[5];
-#pragma unroll
-  for (int o = 0; o < 5; ++o) {
-    X[o] = wrapc(x + o - 2, g.nx);
-    Y[o] = wrapc(y + o - 2, g.ny);
-    Z[o] = wrapc(z + o - 2, g.nz);
-  }
+  const unsigned sides = __ballot_sync(FULL, ok) >> base;
+  const bool open = (sides & 0x3fu) == 0x3fu;
+  RC nh[3] = {(RC)0, (RC)0, (RC)0};
+  if (ok && (sub < 6 || !open)) unit_normal<RC>(g, flags, phi, px, py, pz, nh);
+  const RC own = sub < 2 ? nh[0] : sub < 4 ? nh[1] : nh[2];
   RC div = (RC)0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    RC nh[2][3];
-#pragma unroll
-    for (int sgn = 0; sgn < 2; ++sgn) {
-      // point p = centre + (+1 | -1) e_a, in offset coordinates (2 = centre)
-      int pc[3] = {2, 2, 2};
-      pc[a] += sgn == 0 ? 1 : -1;
-      RC v[3][3][3];  // phi around p, v[dz+1][dy+1][dx+1]
-#pragma unroll
-      for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-        for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-          for (int dx = -1; dx <= 1; ++dx)
-            v[dz + 1][dy + 1][dx + 1] =
-                (RC)phi[X[pc[0] + dx] + g.sx * (Y[pc[1] + dy] + g.ny * Z[pc[2] + dz])];
-      RC n[3];
-#pragma unroll
-      for (int ax = 0; ax < 3; ++ax) {
-        int b = (ax + 1) % 3, cc = (ax + 2) % 3;
-        if (b > cc) { int t = b; b = cc; cc = t; }
-        RC sum = (RC)0;
-#pragma unroll
-        for (int ob = -1; ob <= 1; ++ob)
-#pragma unroll
-          for (int oc = -1; oc <= 1; ++oc) {
-            int op[3] = {0, 0, 0}, om[3] = {0, 0, 0};
-            op[ax] = 1; om[ax] = -1;
-            op[b] += ob; om[b] += ob;
-            op[cc] += oc; om[cc] += oc;
-            const RC w = (RC)((ob == 0 ? 2.0 : 1.0) * (oc == 0 ? 2.0 : 1.0));
-            const RC t = w * (v[op[2] + 1][op[1] + 1][op[0] + 1] - v[om[2] + 1][om[1] + 1][om[0] + 1]);
-            sum = (ob == -1 && oc == -1) ? (RC)0 + t : sum + t;
-          }
-        n[ax] = sum / (RC)32;
-      }
-      // without a branch, so that the loads of all six stencils can be in
-      // flight at once
-      const RC len = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-      const bool tiny = len < (RC)1e-12;
-      const RC l = tiny ? (RC)1 : len;
-      nh[sgn][0] = tiny ? (RC)0 : n[0] / l;
-      nh[sgn][1] = tiny ? (RC)0 : n[1] / l;
-      nh[sgn][2] = tiny ? (RC)0 : n[2] / l;
-    }
-    const RC dd = (RC)0.5 * (nh[0][a] - nh[1][a]);
+    const RC np = __shfl_sync(FULL, own, base + 2 * a), nm = __shfl_sync(FULL, own, base + 2 * a + 1);
+    const RC nc = __shfl_sync(FULL, nh[a], base + 6);
+    const bool okp = (sides >> (2 * a)) & 1u, okm = (sides >> (2 * a + 1)) & 1u;
+    const RC dd = okp && okm ? (RC)0.5 * (np - nm) : okp ? np - nc : okm ? nc - nm : (RC)0;
     div = (a == 0) ? (RC)0 + dd : div + dd;
   }
   return -div;
-}
-
-// true when no cell within distance 2 of (x, y, z) can be a wall or obstacle
-__device__ __forceinline__ bool open_neighbourhood(const Geom& g, int x, int y, int z) {
-  if (g.has_obst) return false;
-  if (!g.periodic[0] && (x < 2 || x > g.nx - 3)) return false;
-  if (!g.periodic[1] && (y < 2 || y > g.ny - 3)) return false;
-  if (!g.periodic[2] && (z < 2 || z > g.nz - 3)) return false;
-  return true;
-}
-
-template <class RC, class PT>
-__device__ inline RC curvature_any(const Geom& g, const uint8_t* flags, const PT* phi, int x,
-                                   int y, int z) {
-  return open_neighbourhood(g, x, y, z) ? curvature_open<RC>(g, phi, x, y, z)
-                                        : curvature<RC>(g, flags, phi, x, y, z);
 }
 
 // ------------------------------------------------------------ refilling
@@ -2179,9 +2110,32 @@ __device__ inline uint8_t iface_class(const Geom& g, const uint8_t* flags, int x
   return 0;
 }
 
+// Interface cells a block of 128 threads takes at a time out of n: 128 where
+// the list is long (one list append per 128 cells: same-address atomics queue
+// up otherwise), down to the 16 cells that its eight-lane groups hold where
+// the list is short, so that it is spread over all SMs.
+__device__ __forceinline__ unsigned cells_per_block(unsigned n) {
+  const unsigned per = ((n + gridDim.x - 1) / gridDim.x + 15u) & ~15u;
+  return per < 16u ? 16u : per > 128u ? 128u : per;
+}
+
+// Curvature of the interface cells cell[0..per) that a block has collected
+// (-1: none), eight lanes each.
+template <class ST>
+__device__ __forceinline__ void curvature_block(const Dev& d, const Geom& g, const int* cell,
+                                                unsigned per) {
+  using R = typename ST::R;
+#pragma unroll 1
+  for (unsigned j = threadIdx.x >> 3; j < per; j += 16u) {
+    const int c = cell[j];
+    const R k = curvature8<R>(g, d.flags, phi_work<R>(d), c);
+    if (c >= 0 && (threadIdx.x & 7) == 0) d.kappa[c] = (double)k;
+  }
+}
+
 template <int Q, class ST>
 __device__ __forceinline__ void classify_body(const Dev& d, const Geom& g, const Phys& p) {
-  using R = typename ST::R;
+  __shared__ int cell[128];
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
   const unsigned a = ctrl->n_if, b = ctrl->n_new, e = ctrl->n_l2i;
@@ -2191,9 +2145,11 @@ __device__ __forceinline__ void classify_body(const Dev& d, const Geom& g, const
   // interface in this one: the next step's list is built here
   // block-uniform loop (the append below is block-wide; 128 threads)
   const unsigned n = a + b + e;
-  for (unsigned base = blockIdx.x * 128u; base < n; base += gridDim.x * 128u) {
+  const bool curved = p.sigma != 0.0;
+  const unsigned per = curved ? cells_per_block(n) : 128u;
+  for (unsigned base = blockIdx.x * per; base < n; base += gridDim.x * per) {
     const unsigned k = base + threadIdx.x;
-    const bool ok = k < n;
+    const bool ok = threadIdx.x < per && k < n;
     const int c = !ok ? 0 : (k < a ? lif[k] : (k < a + b ? d.l_new[k - a] : d.l_l2i[k - a - b]));
     bool is_if = false;
     if (ok) {
@@ -2205,11 +2161,16 @@ __device__ __forceinline__ void classify_body(const Dev& d, const Geom& g, const
         int x, y, z;
         cell_xyz(g, c, x, y, z);
         nf |= iface_class<Q>(g, d.flags, x, y, z);
-        d.kappa[c] = (p.sigma != 0.0) ? (double)curvature_any<R>(g, d.flags, phi_work<R>(d), x, y, z) : 0.0;
+        if (!curved) d.kappa[c] = 0.0;
       }
       d.flags[c] = nf;
     }
-    block_append<128>(is_if, c, &ctrl->n_if_next, lnext);
+    if (curved) cell[threadIdx.x] = is_if ? c : -1;
+    block_append<128>(is_if, c, &ctrl->n_if_next, lnext);  // (synchronises the block)
+    if (curved) {
+      curvature_block<ST>(d, g, cell, per);
+      __syncthreads();  // cell[] is rewritten by the next iteration
+    }
   }
 }
 template <int Q, class ST>
@@ -2220,6 +2181,22 @@ template <int Q, class ST>
 __global__ void __launch_bounds__(128, 4) kb_classify(MemberTable t) {
   FSL_MEMBER(t);
   classify_body<Q, ST>(d, g, p);
+}
+
+// Curvature of every cell of the current step's interface list (initial state).
+template <class ST>
+__global__ void __launch_bounds__(128, 4) k_curvature_list(Dev d, Geom g) {
+  __shared__ int cell[128];
+  const unsigned n = d.ctrl->n_if;
+  const int* lif = list_if(d, d.ctrl->step);
+  const unsigned per = cells_per_block(n);
+  for (unsigned base = blockIdx.x * per; base < n; base += gridDim.x * per) {
+    const unsigned k = base + threadIdx.x;
+    cell[threadIdx.x] = threadIdx.x < per && k < n ? lif[k] : -1;
+    __syncthreads();
+    curvature_block<ST>(d, g, cell, per);
+    __syncthreads();
+  }
 }
 
 
@@ -2460,9 +2437,8 @@ __global__ void k_init_state(Dev d, Geom g, Phys p, int cur, const double* u0, d
   }
 }
 
-template <int Q, class ST>
-__global__ void k_init_classes(Dev d, Geom g, Phys p) {
-  using R = typename ST::R;
+template <int Q>
+__global__ void k_init_classes(Dev d, Geom g) {
   const long long total = g.cells;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < total;
        c += (long long)gridDim.x * blockDim.x) {
@@ -2472,7 +2448,6 @@ __global__ void k_init_classes(Dev d, Geom g, Phys p) {
     const uint8_t fl = d.flags[c];
     if ((fl & F_TYPE) != T_IF) continue;
     d.flags[c] = (uint8_t)((fl & ~(F_NF | F_NE)) | iface_class<Q>(g, d.flags, x, y, z));
-    d.kappa[c] = (p.sigma != 0.0) ? (double)curvature_any<R>(g, d.flags, phi_work<R>(d), x, y, z) : 0.0;
   }
 }
 
@@ -2630,8 +2605,10 @@ struct Kernels {
     k_init_types<<<blocks, 256, 0, s>>>(d, g, d.phinew, d.claim, have_obst);
     k_init_close<Q><<<blocks, 256, 0, s>>>(d, g);
     k_init_state<Q, ST><<<blocks, 256, 0, s>>>(d, g, p, cur, u0, h_ref);
-    k_init_classes<Q, ST><<<blocks, 128, 0, s>>>(d, g, p);
+    k_init_classes<Q><<<blocks, 128, 0, s>>>(d, g);
     k_list_interface<<<blocks, 256, 0, s>>>(d, g);
+    // (k_init_state set every curvature to zero)
+    if (p.sigma != 0.0) k_curvature_list<ST><<<kCellListBlocks, 128, 0, s>>>(d, g);
     if (g.bubbles) return bubble_update<Q>(d, g, p, 1, s);
     return cudaGetLastError();
   }
