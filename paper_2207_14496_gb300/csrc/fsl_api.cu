@@ -716,6 +716,7 @@ struct fsl_adjoint {
   double* dinit = nullptr; // 2 x dense cells: d J / d rho0, d J / d phi0
   std::vector<double> column;
   bool forward_done = false;
+  int flip = 0;            // which of the two adjoint state buffers is the input
 };
 
 extern "C++" {
@@ -759,18 +760,20 @@ AdjFields<R> adjoint_fields(fsl_adjoint* a) {
   const size_t qp = (size_t)h->cfg.lattice * h->g.plane, n = (size_t)h->g.cells;
   R* b = reinterpret_cast<R*>(a->fld);
   AdjFields<R> f;
-  f.lF = b;
-  f.lF0 = b + qp;
-  f.lfin = b + 2 * qp;
   R* cb = b + 4 * qp;
-  f.lM = cb;
-  f.lM0 = cb + n;
-  f.lP = cb + 2 * n;
-  f.lP0 = cb + 3 * n;
+  // the level-t adjoint of one step is the input of the next (earlier) one:
+  // the two sets of fields swap roles
+  const int in = a->flip, out = 1 - a->flip;
+  f.lF = b + in * qp;
+  f.lF0 = b + out * qp;
+  f.lfin = b + 2 * qp;
+  f.lM = cb + in * n;
+  f.lM0 = cb + out * n;
+  f.lP = cb + (2 + in) * n;
+  f.lP0 = cb + (2 + out) * n;
   f.lm1 = cb + 4 * n;
   f.lrhoP = cb + 5 * n;
   f.lmnew = cb + 6 * n;
-  f.lrho = cb + 7 * n;
   f.lbar = cb + 10 * n;  // 4 per cell
   f.lg = cb + 14 * n;    // 3 per cell
   f.acc = a->acc;
@@ -780,15 +783,13 @@ AdjFields<R> adjoint_fields(fsl_adjoint* a) {
 // copy the handle's current state into tape level j
 fsl_status adjoint_record(fsl_adjoint* a, int j, long long step) {
   fsl_handle* h = a->h;
-  const int cur = (int)(step & 1);
-  FSL_CK(cudaMemcpyAsync(a->tF + (size_t)j * align256(a->fbytes), h->d.pdf[cur], a->fbytes,
-                         cudaMemcpyDeviceToDevice, h->stream));
-  FSL_CK(cudaMemcpyAsync(a->tFl + (size_t)j * align256(a->cells), h->d.flags, a->cells,
-                         cudaMemcpyDeviceToDevice, h->stream));
-  FSL_CK(cudaMemcpyAsync(a->tM + (size_t)j * align256(a->cells * 8) / 8, h->d.mass, a->cells * 8,
-                         cudaMemcpyDeviceToDevice, h->stream));
-  FSL_CK(cudaMemcpyAsync(a->tP + (size_t)j * align256(a->cells * 8) / 8, h->d.phi, a->cells * 8,
-                         cudaMemcpyDeviceToDevice, h->stream));
+  // (fbytes is a multiple of 16: planes are padded to 128 elements)
+  k_adj_record<<<4 * 152, 256, 0, h->stream>>>(
+      h->d, (int)(step & 1), (long long)(a->fbytes / 16), (long long)a->cells,
+      reinterpret_cast<uint4*>(a->tF + (size_t)j * align256(a->fbytes)),
+      a->tFl + (size_t)j * align256(a->cells), a->tM + (size_t)j * align256(a->cells * 8) / 8,
+      a->tP + (size_t)j * align256(a->cells * 8) / 8);
+  FSL_CK(cudaGetLastError());
   return FSL_OK;
 }
 
@@ -802,23 +803,16 @@ AdjLevel adjoint_level(const fsl_adjoint* a, int j) {
 }
 
 template <int Q, class ST>
-fsl_status adjoint_step(fsl_adjoint* a, const AdjLevel& L0, const AdjLevel& L1) {
+fsl_status adjoint_step(fsl_adjoint* a, const AdjLevel& L0, const AdjLevel& L1, double dj) {
   using R = typename ST::R;
   fsl_handle* h = a->h;
   AdjFields<R> f = adjoint_fields<R>(a);
-  const int blocks = (int)((a->cells + 255) / 256);
-  k_adj_phi<Q, ST><<<blocks, 256, 0, h->stream>>>(h->g, h->p, L0, L1, f);
-  k_adj_mass<Q, ST><<<blocks, 256, 0, h->stream>>>(h->g, h->p, L0, L1, f);
-  k_adj_refill<Q, ST><<<blocks, 256, 0, h->stream>>>(h->g, h->p, L0, L1, f);
-  k_adj_collide<Q, ST><<<blocks, 256, 0, h->stream>>>(h->g, h->p, L0, L1, f);
-  k_adj_state<Q, ST><<<blocks, 256, 0, h->stream>>>(h->g, h->p, L0, f);
+  const int blocks = (int)((a->cells + kAdjThreads - 1) / kAdjThreads);
+  k_adj_interface<Q, ST><<<blocks, kAdjThreads, 0, h->stream>>>(h->g, h->p, L0, L1, f, dj);
+  k_adj_collide<Q, ST><<<blocks, kAdjThreads, 0, h->stream>>>(h->g, h->p, L0, L1, f);
+  k_adj_state<Q, ST><<<blocks, kAdjThreads, 0, h->stream>>>(h->g, h->p, L0, f);
   FSL_CK(cudaGetLastError());
-  // the level-t adjoint becomes the input of the next (earlier) step
-  const size_t rb = sizeof(R);
-  const size_t qp = (size_t)h->cfg.lattice * h->g.plane;
-  FSL_CK(cudaMemcpyAsync(f.lF, f.lF0, qp * rb, cudaMemcpyDeviceToDevice, h->stream));
-  FSL_CK(cudaMemcpyAsync(f.lM, f.lM0, a->cells * rb, cudaMemcpyDeviceToDevice, h->stream));
-  FSL_CK(cudaMemcpyAsync(f.lP, f.lP0, a->cells * rb, cudaMemcpyDeviceToDevice, h->stream));
+  a->flip = 1 - a->flip;
   return FSL_OK;
 }
 
@@ -828,17 +822,19 @@ fsl_status adjoint_init(fsl_adjoint* a, const AdjLevel& L0) {
   fsl_handle* h = a->h;
   AdjFields<R> f = adjoint_fields<R>(a);
   const size_t dense = (size_t)h->g.nx * h->g.ny * h->g.nz;
-  k_adj_init<Q, ST><<<(unsigned)((a->cells + 255) / 256), 256, 0, h->stream>>>(
+  k_adj_init<Q, ST><<<(unsigned)((a->cells + kAdjThreads - 1) / kAdjThreads), kAdjThreads, 0,
+                      h->stream>>>(
       h->g, h->p, L0, f, h->h_ref, a->dinit, a->dinit + dense);
   FSL_CK(cudaGetLastError());
   return FSL_OK;
 }
 
-fsl_status adjoint_dispatch_step(fsl_adjoint* a, const AdjLevel& L0, const AdjLevel& L1) {
+fsl_status adjoint_dispatch_step(fsl_adjoint* a, const AdjLevel& L0, const AdjLevel& L1,
+                                 double dj) {
   const int q = a->h->cfg.lattice;
   if (a->h->cfg.precision == FSL_FP64)
-    return q == 19 ? adjoint_step<19, SF64>(a, L0, L1) : adjoint_step<27, SF64>(a, L0, L1);
-  return q == 19 ? adjoint_step<19, SF32>(a, L0, L1) : adjoint_step<27, SF32>(a, L0, L1);
+    return q == 19 ? adjoint_step<19, SF64>(a, L0, L1, dj) : adjoint_step<27, SF64>(a, L0, L1, dj);
+  return q == 19 ? adjoint_step<19, SF32>(a, L0, L1, dj) : adjoint_step<27, SF32>(a, L0, L1, dj);
 }
 
 fsl_status adjoint_dispatch_init(fsl_adjoint* a, const AdjLevel& L0) {
@@ -931,8 +927,7 @@ fsl_status fsl_adjoint_backward(fsl_adjoint* a, const double* dj_dcolumn, double
   const size_t dense = (size_t)h->g.nx * h->g.ny * h->g.nz;
   FSL_CK(cudaMemsetAsync(a->fld, 0, rb * (4 * qp + 17 * a->cells), h->stream));
   FSL_CK(cudaMemsetAsync(a->acc, 0, 8 * sizeof(double), h->stream));
-  double* lP_dbl = rb == 8 ? reinterpret_cast<double*>(a->fld) + 4 * qp + 2 * a->cells : nullptr;
-  float* lP_flt = rb == 4 ? reinterpret_cast<float*>(a->fld) + 4 * qp + 2 * a->cells : nullptr;
+  a->flip = 0;
   for (int k = a->nseg - 1; k >= 0; --k) {
     const int t0 = k * a->every;
     const int len = std::min(a->every, a->nsteps - t0);
@@ -948,10 +943,8 @@ fsl_status fsl_adjoint_backward(fsl_adjoint* a, const double* dj_dcolumn, double
       if (st != FSL_OK) return st;
     }
     for (int j = len; j >= 1; --j) {
-      k_adj_observe<<<(h->g.ny * h->g.nz + 255) / 256, 256, 0, h->stream>>>(
-          h->g, dj_dcolumn[t0 + j - 1], lP_dbl, lP_flt);
-      FSL_CK(cudaGetLastError());
-      st = adjoint_dispatch_step(a, adjoint_level(a, j - 1), adjoint_level(a, j));
+      st = adjoint_dispatch_step(a, adjoint_level(a, j - 1), adjoint_level(a, j),
+                                 dj_dcolumn[t0 + j - 1]);
       if (st != FSL_OK) return st;
     }
   }
