@@ -199,8 +199,8 @@ int fsl_launches_per_step(const fsl_handle* h);
  *     packed FP32 with at most 128, 96 and 80 registers per thread (four,
  *     five and six blocks per SM); PAIR_R128 collides them one after the
  *     other (128 registers);
- *   TMA: persistent, tiles of 256 cells with liquid (listed by a pre-pass)
- *     staged in shared memory by bulk copies through a ring of
+ *   TMA: persistent, tiles of 256 cells with liquid (listed by a pre-pass; of
+ *     several whole rows where a row has at most 128 cells) staged in shared memory by bulk copies through a ring of
  *     mbarrier-guarded stages, one producer warp and four consumer warps;
  *   QUAD_64 (16-bit storages only): four cells per thread, 64 threads per
  *     block, one 8-byte load per direction kept packed until the collision;
@@ -227,8 +227,10 @@ int fsl_launches_per_step(const fsl_handle* h);
  *     on one cell in FP32, at most 64 (CELL) or 80 (CELL_R80) registers;
  *   TMA_R96 (16-bit storages only): as TMA with three stages and four blocks
  *     per SM (at most 102 registers), sixteen consumer warps per SM.
- * DEFAULT is PAIR_R128; the Python autotuner
- * (paper_2207_14496_gb300.autotune) measures the variants instead.
+ * DEFAULT picks by the domain: TMA from 2.5 million (padded) cells on and in
+ * domains with obstacles, SEG_R128 from 200,000 cells on, PAIR_R128 below; the
+ * Python autotuner (paper_2207_14496_gb300.autotune) measures the variants
+ * instead.
  * fsl_set_variant drops captured step graphs; FSL_ERR_ARG for an unknown
  * variant and for QUAD_64, PAIR_PIPE, CPA_R96 or TMA_R96 with FP32 storage. */
 enum { FSL_VARIANT_DEFAULT = 0, FSL_VARIANT_PAIR = 1, FSL_VARIANT_PAIR_R128 = 2,

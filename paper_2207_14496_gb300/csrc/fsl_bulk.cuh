@@ -1,14 +1,17 @@
 // Bulk pass of the 16/32-bit path, staged through shared memory by the TMA.
 //
 // k_tiles lists, at the start of a step, the tiles (256 cells along x of one
-// (y, z) row) that hold liquid cells.
+// (y, z) row) that hold liquid cells; for rows of at most 128 cells
+// k_row_tiles lists tiles of several whole rows of a z-plane.
 //
 // k_stream_collide_bulk is persistent and warp-specialised.  Its producer warp
 // walks the CTA's share of the tile list and, for each tile, issues Q + 1
 // one-dimensional bulk copies (cp.async.bulk, the untiled TMA form) into a
 // ring of shared-memory stages: for each direction i the 256 + 2*8 stored
 // values of plane i on the row (y - c_iy, z - c_iz) that the tile pulls
-// from (clipped to the row), and the tile's 256 flag bytes.  Each copy group
+// from (clipped to the row), and the tile's 256 flag bytes.  The source rows
+// of a tile of several rows are contiguous but for the row beyond an end of
+// the plane, which takes a copy of its own.  Each copy group
 // completes on the stage's "full" mbarrier.  Four consumer warps, two
 // neighbouring cells per thread, wait on "full", pull their 27 (or 19) value
 // pairs out of shared memory, collide both cells in packed FP32 (collide_v)
@@ -89,6 +92,66 @@ struct BulkRing {
   static constexpr size_t bytes = stages * stage_bytes + 2 * stages * 8 + 16 * stages + 16;
 };
 
+// whether a 16-byte word of flag bytes holds a liquid cell
+__device__ __forceinline__ bool any_liquid(const uint4& v) {
+  const unsigned u[4] = {v.x, v.y, v.z, v.w};
+  bool liq = false;
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    // a byte whose type bits are T_LIQ: (b & 3) ^ 2 == 0
+    const unsigned t = (u[h] & 0x03030303u) ^ 0x02020202u;
+    liq |= ((t - 0x01010101u) & ~t & 0x80808080u) != 0u;
+  }
+  return liq;
+}
+
+// Tiles of whole rows for rows of at most half a tile: rows per tile (the last
+// tile of a plane may hold fewer) and tiles per plane.  rows = 1: the domain
+// is cut into tiles of one row instead.
+struct RowTiles {
+  int rows, per;
+};
+inline RowTiles row_tiles(const Geom& g) {
+  RowTiles t;
+  t.rows = g.sx <= kBulkTX / 2 && g.ny > 1 ? (kBulkTX / g.sx < g.ny ? kBulkTX / g.sx : g.ny) : 1;
+  t.per = (g.ny + t.rows - 1) / t.rows;
+  return t;
+}
+
+// List the row tiles with liquid cells: a half-warp reads a tile's flag
+// bytes, contiguous, 16 per lane; a block takes 16 tiles at a time, 64 in
+// all, and appends what it found with one atomic (the order of the list does
+// not matter to its consumers).
+static __global__ void __launch_bounds__(256) k_row_tiles(Dev d, Geom g, RowTiles rt) {
+  __shared__ int found[64];
+  __shared__ int nfound;
+  __shared__ unsigned base;
+  Ctrl* ctrl = d.ctrl;
+  if (frozen(ctrl)) return;
+  if (threadIdx.x == 0) nfound = 0;
+  __syncthreads();
+  const int sub = threadIdx.x & 15, grp = threadIdx.x >> 4;
+  const unsigned half = 0xffffu << (threadIdx.x & 16);
+  const int ntiles = rt.per * g.nz;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int k = blockIdx.x * 64 + 16 * j + grp;
+    bool liq = false;
+    if (k < ntiles) {
+      const int y0 = (k % rt.per) * rt.rows;
+      const int n = (g.ny - y0 < rt.rows ? g.ny - y0 : rt.rows) * g.sx;
+      const uint8_t* f = d.flags + ((long long)(k / rt.per) * g.ny + y0) * g.sx;
+      if (16 * sub < n) liq = any_liquid(*reinterpret_cast<const uint4*>(f + 16 * sub));
+    }
+    const bool any = (__ballot_sync(0xffffffffu, liq) & half) != 0u;
+    if (any && sub == 0) found[atomicAdd(&nfound, 1)] = k;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) base = nfound ? atomicAdd(&ctrl->n_tiles, (unsigned)nfound) : 0u;
+  __syncthreads();
+  if ((int)threadIdx.x < nfound) d.l_tiles[base + threadIdx.x] = found[threadIdx.x];
+}
+
 // List the tiles (TX cells along x of one row) with liquid cells.  One thread
 // per tile reads the tile's flag bytes in 16-byte words; a block's tiles are
 // ranked by warp ballots and appended with one atomic per block (the order of
@@ -111,14 +174,7 @@ __device__ __forceinline__ void tiles_body(const Dev& d, const Geom& g, int ntx)
     const int n = (g.sx - x0 < TX ? g.sx - x0 : TX) / 16;  // 16-byte words in the padded row
     const uint4* w = reinterpret_cast<const uint4*>(d.flags + row * g.sx + x0);
     for (int q = 0; q < n && !liq; ++q) {
-      const uint4 v = w[q];
-      const unsigned u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        // a byte whose type bits are T_LIQ: (b & 3) ^ 2 == 0
-        const unsigned t = (u[h] & 0x03030303u) ^ 0x02020202u;
-        liq |= ((t - 0x01010101u) & ~t & 0x80808080u) != 0u;
-      }
+      liq |= any_liquid(w[q]);
     }
   }
   const unsigned m = __ballot_sync(0xffffffffu, liq);
@@ -156,10 +212,10 @@ __global__ void __launch_bounds__(256) kb_tiles(MemberTable t) {
 // out of shared memory, both cells collide in packed FP32 and the results go
 // to HBM.  The periodic wrap along x at the two row ends: wrap = 0, read from
 // HBM; 1, the stage holds the wrapped halos; 2, the stage holds the whole row
-// (x0 = 0, nx <= the tile width) and the value comes from its other end.
-// Liquid cells next to a domain wall (no obstacle cell, no free-slip wall)
-// take the halfway bounce-back value for the directions that cross the wall;
-// next to an obstacle or a free-slip wall the per-direction path reads HBM.
+// and the value comes from its other end.
+// Liquid cells next to a wall or obstacle take the halfway bounce-back value
+// for the directions whose source is solid; in domains with free-slip walls
+// the per-direction path reads HBM.
 // Returns whether a liquid cell reached |u|^2 >= 1/3.
 template <int Q, class ST>
 __device__ __forceinline__ bool bulk_pair(const typename ST::T* __restrict__ A,
@@ -219,17 +275,13 @@ __device__ __forceinline__ bool bulk_pair(const typename ST::T* __restrict__ A,
   }
   const long long c = (long long)row * g.sx + xa;
   const bool near0 = liq0 && (fl0 & F_NEAR_OBST), near1 = liq1 && (fl1 & F_NEAR_OBST);
-  if ((near0 || near1) && !g.has_obst && !g.free_slip) {
-    const bool wl0 = !g.periodic[0] && xa == 0, wr0 = !g.periodic[0] && xa + 1 >= g.nx;
-    const bool wr1 = !g.periodic[0] && xa + 2 >= g.nx;
-    const bool ylo = !g.periodic[1] && y == 0, yhi = !g.periodic[1] && y == g.ny - 1;
-    const bool zlo = !g.periodic[2] && z == 0, zhi = !g.periodic[2] && z == g.nz - 1;
+  if ((near0 || near1) && !g.free_slip) {
+    const unsigned m0 = near0 ? solid_sources<Q>(d.flags, g, xa, y, z) : 0u;
+    const unsigned m1 = near1 ? solid_sources<Q>(d.flags, g, xa + 1, y, z) : 0u;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-      const int cx = dir_c(i, 0), cy = dir_c(i, 1), cz = dir_c(i, 2);
-      const bool yz = (cy == 1 && ylo) || (cy == -1 && yhi) || (cz == 1 && zlo) || (cz == -1 && zhi);
-      if (near0 && (yz || (cx == 1 && wl0) || (cx == -1 && wr0))) f[i].x = ST::ld1(A + opp(i) * P + c);
-      if (near1 && (yz || (cx == -1 && wr1))) f[i].y = ST::ld1(A + opp(i) * P + c + 1);
+      if ((m0 >> i) & 1u) f[i].x = ST::ld1(A + opp(i) * P + c);
+      if ((m1 >> i) & 1u) f[i].y = ST::ld1(A + opp(i) * P + c + 1);
     }
   } else if (near0 || near1) {
 #pragma unroll
@@ -260,16 +312,20 @@ __device__ __forceinline__ bool bulk_pair(const typename ST::T* __restrict__ A,
   return (liq0 && !(usq.x < (float)(1.0 / 3.0))) || (liq1 && !(usq.y < (float)(1.0 / 3.0)));
 }
 
-template <int Q, class ST, int NS, int MINB>
+// MULTI: tiles of rt.rows whole rows of a plane (rows of at most 128 cells);
+// else tiles of 256 cells of one row.  A 64-cell row fills only a quarter of
+// a one-row tile's lanes: 64x64x640, D3Q19, FP32, tube of obstacles, 278 us with one-row tiles' pair kernel, 106 us here.
+template <int Q, class ST, int NS, int MINB, bool MULTI>
 __global__ void __launch_bounds__(kBulkThreads, MINB)
-    k_stream_collide_bulk(Dev d, Geom g, Phys p, int ntx) {
+    k_stream_collide_bulk(Dev d, Geom g, Phys p, int ntx, RowTiles rt) {
   using T = typename ST::T;
   using RING = BulkRing<Q, ST, NS>;
   constexpr int D = RING::stages;
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + D * RING::stage_bytes);
   uint64_t* empty = full + D;
-  int4* tile_of = reinterpret_cast<int4*>(empty + D);  // (x0, row, y, z) held by each stage
+  // (x0, row, y, z) held by each stage; MULTI: (rows, first row, first y, z)
+  int4* tile_of = reinterpret_cast<int4*>(empty + D);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tile_of + D);
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
@@ -312,13 +368,46 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
         break;
       }
       const int k = d.l_tiles[ti];
+      unsigned char* stage = smem + (size_t)s * RING::stage_bytes;
+      if constexpr (MULTI) {
+        const int z = k / rt.per, y0 = (k % rt.per) * rt.rows;
+        const int R = g.ny - y0 < rt.rows ? g.ny - y0 : rt.rows;
+        const unsigned row_bytes = (unsigned)(g.sx * sizeof(T));
+        if (lane == 0) {
+          tile_of[s] = make_int4(R, z * g.ny + y0, y0, z);
+          mbar_expect_tx(&full[s], R * row_bytes * Q + (unsigned)(R * g.sx));
+        }
+        __syncwarp();
+        if (lane < Q) {
+          int zs = z - rc(lane, 2);
+          zs = zs < 0 ? (g.periodic[2] ? g.nz - 1 : z) : (zs >= g.nz ? (g.periodic[2] ? 0 : z) : zs);
+          const T* plane = A + lane * P + (long long)g.sx * g.ny * zs;
+          T* dst = reinterpret_cast<T*>(stage) + kBulkHalo + (size_t)lane * kBulkSeg;
+          // source rows ys .. ys + R - 1; the one beyond an end of the plane is
+          // at its other end (beyond a wall any row will do: the cells there
+          // take the bounce-back value)
+          const int ys = y0 - rc(lane, 1);
+          const bool below = ys < 0, above = ys + R > g.ny;
+          const int first = below ? 1 : 0, n = R - (below || above ? 1 : 0);
+          if (below || above)
+            bulk_copy_g2s(dst + (below ? 0 : R - 1) * g.sx,
+                          plane + (long long)g.sx * (below ? g.ny - 1 : 0), row_bytes, &full[s]);
+          if (n > 0)
+            bulk_copy_g2s(dst + first * g.sx, plane + (long long)g.sx * (ys + first), n * row_bytes,
+                          &full[s]);
+        } else if (lane == Q) {
+          bulk_copy_g2s(stage + RING::pdf_bytes, d.flags + (long long)(z * g.ny + y0) * g.sx,
+                        (unsigned)(R * g.sx), &full[s]);
+        }
+        ++issued;
+        continue;
+      }
       const int x0 = (k % ntx) * kBulkTX;
       const int row = k / ntx;
       const int lo = x0 - kBulkHalo > 0 ? x0 - kBulkHalo : 0;
       const int hi = x0 + kBulkTX + kBulkHalo < g.sx ? x0 + kBulkTX + kBulkHalo : g.sx;
       const unsigned bytes = (unsigned)((hi - lo) * sizeof(T));
       const unsigned fbytes = (unsigned)(g.sx - x0 < kBulkTX ? g.sx - x0 : kBulkTX);
-      unsigned char* stage = smem + (size_t)s * RING::stage_bytes;
       if (lane == 0) {
         // published to the consumers by the arrive below
         tile_of[s] = make_int4(x0, row, row % g.ny, row / g.ny);
@@ -352,6 +441,7 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
   // ---------------- consumer warps: two cells (2t, 2t + 1) of the tile per thread
   const LesLp les = LesLp::of(p);
   const int t = threadIdx.x;
+  const int rt_r = MULTI ? 2 * t / g.sx : 0;  // row of the tile the thread's cells lie in
   bool bad = false;
   for (int j = 0;; ++j) {
     const int ti = blockIdx.x + j * gridDim.x;
@@ -368,13 +458,21 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
     }
     const unsigned char* stage = smem + (size_t)s * RING::stage_bytes;
     const int4 tc = tile_of[s];
-    const int xa = tc.x + 2 * t;
     const uchar2 f2 = *reinterpret_cast<const uchar2*>(stage + RING::pdf_bytes + 2 * t);
-    const uint8_t fl0 = xa < g.nx ? f2.x : (uint8_t)T_GAS;
-    const uint8_t fl1 = xa + 1 < g.nx ? f2.y : (uint8_t)T_GAS;
-    bad |= bulk_pair<Q, ST>(A, B, reinterpret_cast<const T*>(stage), kBulkSeg, kBulkHalo + 2 * t,
-                            xa, tc.y, tc.z, tc.w, fl0, fl1, d, g, p, les,
-                            (tc.x == 0 && g.nx <= kBulkTX) ? 2 : 0);
+    if constexpr (MULTI) {
+      // (the cells of a row's padding hold the gas type)
+      if (rt_r < tc.x)
+        bad |= bulk_pair<Q, ST>(A, B, reinterpret_cast<const T*>(stage), kBulkSeg,
+                                kBulkHalo + 2 * t, 2 * t - rt_r * g.sx, tc.y + rt_r, tc.z + rt_r,
+                                tc.w, f2.x, f2.y, d, g, p, les, 2);
+    } else {
+      const int xa = tc.x + 2 * t;
+      const uint8_t fl0 = xa < g.nx ? f2.x : (uint8_t)T_GAS;
+      const uint8_t fl1 = xa + 1 < g.nx ? f2.y : (uint8_t)T_GAS;
+      bad |= bulk_pair<Q, ST>(A, B, reinterpret_cast<const T*>(stage), kBulkSeg, kBulkHalo + 2 * t,
+                              xa, tc.y, tc.z, tc.w, fl0, fl1, d, g, p, les,
+                              (tc.x == 0 && g.nx <= kBulkTX) ? 2 : 0);
+    }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
   }

@@ -727,6 +727,49 @@ __device__ __noinline__ float pull_one(const typename ST::T* __restrict__ A, lon
   return ST::ld1(A + dir * plane + n);
 }
 
+// the directions with velocity component v along axis a, as a bit mask
+template <int Q>
+__host__ __device__ constexpr unsigned dirs_with(int a, int v) {
+  unsigned m = 0;
+  for (int i = 1; i < Q; ++i)
+    if (dir_c(i, a) == v) m |= 1u << i;
+  return m;
+}
+// Obstacle sources of cell (x, y, z): bit i for a source x - c_i that is an
+// obstacle cell.  All flag bytes are loaded together; out of line (the rare
+// cells next to an obstacle), with a mask in place of an array of values, so
+// that the fast path pays no registers or stack for it.
+template <int Q>
+__device__ __noinline__ unsigned obstacle_sources(const uint8_t* flags, const Geom& g, int x, int y,
+                                                  int z) {
+  Nbr nb;
+  nb.setup(g, x, y, z);
+  const int c = nb.in(0, 0, 0);
+  unsigned m = 0u;
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const int n = nb.at(-dir_c(i, 0), -dir_c(i, 1), -dir_c(i, 2));
+    if ((flags[n >= 0 ? n : c] & F_TYPE) == T_OBST) m |= 1u << i;
+  }
+  return m;
+}
+// Solid sources of the liquid cell (x, y, z) in a domain without free-slip
+// walls: bit i where the PDF f_i comes from beyond a no-slip wall or from an
+// obstacle, so that f*_(opp i) of the cell itself bounces back into it.  One
+// mask in place of a flag load and then a value load per direction
+// (pull_near): a 64x64x640 tube of obstacles, D3Q19, FP32, one cell pair per
+// thread: 281 -> 132 us.
+template <int Q>
+__device__ __forceinline__ unsigned solid_sources(const uint8_t* flags, const Geom& g, int x, int y,
+                                                  int z) {
+  unsigned m = 0u;
+  if (!g.periodic[0]) m |= (x == 0 ? dirs_with<Q>(0, 1) : 0u) | (x == g.nx - 1 ? dirs_with<Q>(0, -1) : 0u);
+  if (!g.periodic[1]) m |= (y == 0 ? dirs_with<Q>(1, 1) : 0u) | (y == g.ny - 1 ? dirs_with<Q>(1, -1) : 0u);
+  if (!g.periodic[2]) m |= (z == 0 ? dirs_with<Q>(2, 1) : 0u) | (z == g.nz - 1 ? dirs_with<Q>(2, -1) : 0u);
+  if (g.has_obst) m |= obstacle_sources<Q>(flags, g, x, y, z);
+  return m;
+}
+
 template <int Q>
 __device__ __forceinline__ float collide_lp(const float* f, float* o, float lamE, float lamO,
                                             float pe, float po, float gx, float gy, float gz,
@@ -800,35 +843,27 @@ __device__ __forceinline__ bool pair_update(const Dev& d, const Geom& g, const P
       if (wrap0) f[i].x = ST::ld1(base);
     }
   }
-  // cells with a wall or obstacle in their stencil.  Domain walls only (no
-  // obstacle cell, no free-slip wall): a PDF whose source lies beyond a wall
+  // cells with a wall or obstacle in their stencil: a PDF whose source is solid
   // is the cell's own f*_(opp i) (halfway bounce-back), every other pulled
-  // value above came from the right row already.  Otherwise the general
-  // per-direction path, out of line.
-  const bool walls_only = !g.has_obst && !g.free_slip;
-  if (walls_only && ((liq0 && (fl0 & F_NEAR_OBST)) || (liq1 && (fl1 & F_NEAR_OBST)))) {
-    const bool wl0 = !g.periodic[0] && x0 == 0, wr1 = !g.periodic[0] && x0 + 2 >= g.nx;
-    const bool wr0 = !g.periodic[0] && x0 + 1 >= g.nx;
-    const bool ylo = !g.periodic[1] && y == 0, yhi = !g.periodic[1] && y == g.ny - 1;
-    const bool zlo = !g.periodic[2] && z == 0, zhi = !g.periodic[2] && z == g.nz - 1;
+  // value above came from the right cell already; free-slip walls take the
+  // general per-direction path, out of line
+  const bool near0 = liq0 && (fl0 & F_NEAR_OBST), near1 = liq1 && (fl1 & F_NEAR_OBST);
+  if ((near0 || near1) && !g.free_slip) {
+    const unsigned m0 = near0 ? solid_sources<Q>(d.flags, g, x0, y, z) : 0u;
+    const unsigned m1 = near1 ? solid_sources<Q>(d.flags, g, x0 + 1, y, z) : 0u;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-      const int cx = dir_c(i, 0), cy = dir_c(i, 1), cz = dir_c(i, 2);
-      // the source x - c_i crosses a wall in y or z (both cells), or in x
-      const bool yz = (cy == 1 && ylo) || (cy == -1 && yhi) || (cz == 1 && zlo) || (cz == -1 && zhi);
-      const bool c0 = yz || (cx == 1 && wl0) || (cx == -1 && wr0);
-      const bool c1 = yz || (cx == -1 && wr1);
-      if (liq0 && (fl0 & F_NEAR_OBST) && c0) f[i].x = ST::ld1(A + opp(i) * P + row + x0);
-      if (liq1 && (fl1 & F_NEAR_OBST) && c1) f[i].y = ST::ld1(A + opp(i) * P + row + x0 + 1);
+      if ((m0 >> i) & 1u) f[i].x = ST::ld1(A + opp(i) * P + row + x0);
+      if ((m1 >> i) & 1u) f[i].y = ST::ld1(A + opp(i) * P + row + x0 + 1);
     }
-  } else if ((liq0 && (fl0 & F_NEAR_OBST)) || (liq1 && (fl1 & F_NEAR_OBST))) {
+  } else if (near0 || near1) {
     float t[Q];
-    if (liq0 && (fl0 & F_NEAR_OBST)) {
+    if (near0) {
       pull_near<Q, ST>(A, P, d.flags, g, x0, y, z, t);
 #pragma unroll
       for (int i = 0; i < Q; ++i) f[i].x = t[i] * S;
     }
-    if (liq1 && (fl1 & F_NEAR_OBST)) {
+    if (near1) {
       pull_near<Q, ST>(A, P, d.flags, g, x0 + 1, y, z, t);
 #pragma unroll
       for (int i = 0; i < Q; ++i) f[i].y = t[i] * S;
@@ -2703,34 +2738,53 @@ struct Kernels {
       return g.variant;
     if ((g.variant == 5 || g.variant == 7 || g.variant == 11 || g.variant == 16) && half)
       return g.variant;
+    // FSL_VARIANT_DEFAULT, by measured step times (us, pair_r128 / seg_r128 /
+    // tma; D3Q27 drop impacts n^3, D3Q19 dam breaks, tubes of obstacles):
+    //   large domains fill the TMA ring of every SM: 200^3 FP16 332 / 314 / 243,
+    //   FP32 416 / 358 / 273; 160^3 FP16 217 / 219 / 209, FP32 262 / 242 / 222;
+    //   obstacles: 64x64x640 FP32 382 / 379 / 364, 32x32x320 FP16 177 / 177 / 169
+    if (g.has_obst || g.cells >= 2500000) return 4;
+    //   medium ones gain from walking the list of liquid segments: 512x256x16
+    //   FP32 116 / 100 / 116, 100^3 FP32 142 / 126 / 140, FP16 122 / 110 / 122
+    if (g.cells >= 200000) return 13;
+    //   in small ones every warp runs at once: 64x64x4 FP32 69 / 71 / 71
     return 2;
   }
   // variants that walk the list of liquid tiles of 256 cells
   static bool uses_tiles256(int v) {
     return v == 4 || v == 9 || v == 10 || v == 11 || v == 16;
   }
+  // of these, those that take tiles of several rows in narrow domains
+  static bool uses_row_tiles(int v) { return v == 4 || v == 16; }
   // variants that walk the list of liquid segments of 64 cells
   static bool uses_segments64(int v) { return v == 6 || (v >= 12 && v <= 15); }
   // persistent TMA pipeline (one producer warp, four consumer warps) with NS
   // stages and at least MINB blocks per SM
   template <int NS, int MINB>
   static cudaError_t launch_tma(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
+    const RowTiles rt = row_tiles(g);
+    if (rt.rows > 1) return launch_tma_as<NS, MINB, true>(d, g, p, rt, s);
+    return launch_tma_as<NS, MINB, false>(d, g, p, rt, s);
+  }
+  template <int NS, int MINB, bool MULTI>
+  static cudaError_t launch_tma_as(const Dev& d, const Geom& g, const Phys& p, const RowTiles& rt,
+                                   cudaStream_t s) {
     static int grid = 0;
     constexpr size_t smem = BulkRing<Q, ST, NS>::bytes;
+    auto* kernel = k_stream_collide_bulk<Q, ST, NS, MINB, MULTI>;
     if (grid == 0) {
-      cudaError_t e = cudaFuncSetAttribute(k_stream_collide_bulk<Q, ST, NS, MINB>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaError_t e =
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
       int per_sm = 0, dev = 0, sms = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_bulk<Q, ST, NS, MINB>,
-                                                        kBulkThreads, smem);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBulkThreads, smem);
       if (e != cudaSuccess) return e;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       grid = (per_sm > 0 ? per_sm : 1) * sms;
     }
     const int ntx = (g.nx + kBulkTX - 1) / kBulkTX;
-    k_stream_collide_bulk<Q, ST, NS, MINB><<<grid, kBulkThreads, smem, s>>>(d, g, p, ntx);
+    kernel<<<grid, kBulkThreads, smem, s>>>(d, g, p, ntx, rt);
     return cudaGetLastError();
   }
   // persistent cp.async pipeline with S stages and at least MINB blocks per SM
@@ -2756,6 +2810,11 @@ struct Kernels {
   }
   static cudaError_t pre_bulk(const Dev& d, const Geom& g, const Phys&, cudaStream_t s) {
     if constexpr (ST::kShift) {
+      const RowTiles rt = row_tiles(g);
+      if (uses_row_tiles(variant_of(g)) && rt.rows > 1) {
+        k_row_tiles<<<(unsigned)((rt.per * g.nz + 63) / 64), 256, 0, s>>>(d, g, rt);
+        return cudaGetLastError();
+      }
       if (uses_tiles256(variant_of(g))) {
         const int ntx = (g.nx + kBulkTX - 1) / kBulkTX;
         const long long ntiles = (long long)ntx * g.ny * g.nz;
