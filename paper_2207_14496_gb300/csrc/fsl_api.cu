@@ -255,6 +255,7 @@ struct fsl_handle {
   bool ready;
   int trace_every;
   std::map<int, cudaGraphExec_t> graphs;
+  int since_sort = 0;  // steps since the interface list was in memory order
   unsigned gen = 0;  // bumped whenever captured launch parameters may change
   char* base = nullptr;         // start of the workspace
   Aux aux = {nullptr, nullptr, nullptr};  // side stream of the interface pass
@@ -279,6 +280,21 @@ fsl_status copy_field(fsl_handle* h, const void* dev, size_t elem, void* host) {
 }
 
 const size_t kGraphChunk = 64;
+// The interface list is put back into memory order (k_sort_interface) when
+// this many steps have passed: 6 us of a 256^3 domain per chunk of 64 steps.
+const int kSortEvery = 48;
+
+// queue k_sort_interface on `s` if it is due, and count the coming steps
+cudaError_t sort_if_due(fsl_handle* h, int steps, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  if (h->since_sort >= kSortEvery) {
+    k_sort_interface<<<(unsigned)((h->g.cells + kSortCells - 1) / kSortCells), 256, 0, s>>>(h->d, h->g);
+    e = cudaGetLastError();
+    h->since_sort = 0;
+  }
+  h->since_sort += steps;
+  return e;
+}
 
 }  // namespace
 
@@ -411,7 +427,10 @@ fsl_status fsl_step(fsl_handle* h, int nsteps) {
   if (h->stream) FSL_CK(cudaStreamIsCapturing(h->stream, &cs));
   if (!h->stream || cs != cudaStreamCaptureStatusNone) {
     // legacy default stream (not capturable) or a capture owned by the caller
-    for (int k = 0; k < nsteps; ++k) FSL_CK(h->L->step(h->d, h->g, h->p, h->stream, h->aux));
+    for (int k = 0; k < nsteps; ++k) {
+      FSL_CK(sort_if_due(h, 1, h->stream));
+      FSL_CK(h->L->step(h->d, h->g, h->p, h->stream, h->aux));
+    }
     return FSL_OK;
   }
   int left = nsteps;
@@ -432,6 +451,7 @@ fsl_status fsl_step(fsl_handle* h, int nsteps) {
       if (ie != cudaSuccess) return cuda_fail(ie, "cudaGraphInstantiate");
       it = h->graphs.emplace(chunk, exec).first;
     }
+    FSL_CK(sort_if_due(h, chunk, h->stream));
     FSL_CK(cudaGraphLaunch(it->second, h->stream));
     left -= chunk;
   }
@@ -1146,6 +1166,7 @@ fsl_status fsl_batch_step(fsl_batch* b, int nsteps) {
       if (st != FSL_OK) return st;
       it = b->graphs.emplace(c, exec).first;
     }
+    for (fsl_handle* h : b->hs) FSL_CK(sort_if_due(h, c, b->stream));
     FSL_CK(cudaGraphLaunch(it->second, b->stream));
     left -= c;
   }

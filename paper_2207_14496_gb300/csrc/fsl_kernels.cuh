@@ -2311,6 +2311,70 @@ static __global__ void k_list_interface(Dev d, Geom g) {
   }
 }
 
+// The interface list of the current step put back into memory order.  Every
+// step appends the next list block by block in the order in which the blocks
+// arrive, and new cells at the end, so over hundreds of steps the cells that a
+// warp takes from the list drift apart in memory and its gathers (108 per cell
+// in the interface pass, 162 in classify) fall apart into one sector per lane.
+// Nothing depends on the order but the speed.  Each block lists kSortCells
+// consecutive cells in order with one atomic; n_if_next and end_blocks, zero
+// between steps, count, and the last block clears them again (the count is the
+// n_if that the step already has).
+constexpr int kSortCells = 256 * 64;
+__device__ __forceinline__ void sort_interface_body(const Dev& d, const Geom& g) {
+  __shared__ unsigned warp_n[8];
+  __shared__ unsigned base;
+  Ctrl* ctrl = d.ctrl;
+  if (frozen(ctrl)) return;
+  const long long c0 = blockIdx.x * (long long)kSortCells + 64 * threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long mask = 0;  // interface cells among the thread's 64
+  if (c0 < g.cells) {
+    // rows are padded to multiples of 32 cells: two 16-byte words at a time
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (c0 + 16 * q >= g.cells) break;
+      const uint4 v = *reinterpret_cast<const uint4*>(d.flags + c0 + 16 * q);
+      const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int h = 0; h < 16; ++h)
+        if (((u[h / 4] >> (8 * (h % 4))) & F_TYPE) == T_IF) mask |= 1ull << (16 * q + h);
+    }
+  }
+  const unsigned n = (unsigned)__popcll(mask);
+  unsigned before = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(0xffffffffu, before, o);
+    if (lane >= o) before += t;
+  }
+  if (lane == 31) warp_n[warp] = before;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned t = 0;
+    for (int w = 0; w < 8; ++w) {
+      const unsigned k = warp_n[w];
+      warp_n[w] = t;
+      t += k;
+    }
+    base = t ? atomicAdd(&ctrl->n_if_next, t) : 0u;
+  }
+  __syncthreads();
+  int* out = list_if(d, ctrl->step) + base + warp_n[warp] + before - n;
+  for (; mask; mask &= mask - 1) *out++ = (int)(c0 + __ffsll(mask) - 1);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&ctrl->end_blocks, 1u) == gridDim.x - 1) {
+      ctrl->n_if_next = 0;
+      ctrl->end_blocks = 0;
+    }
+  }
+}
+static __global__ void __launch_bounds__(256) k_sort_interface(Dev d, Geom g) {
+  sort_interface_body(d, g);
+}
+
 // Deterministic block reduction helpers (fixed tree order).
 template <int NT>
 __device__ inline double block_sum(double v, double* sh) {
