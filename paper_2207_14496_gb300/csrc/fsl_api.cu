@@ -8,7 +8,10 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <thread>
 #include <vector>
+
+#include <unistd.h>
 
 #include "fsl.h"
 #include "fsl_kernels.cuh"
@@ -233,6 +236,23 @@ __global__ void k_count_types(Dev d, Geom g, unsigned long long* out) {
   atomicAdd(&out[1], itf);
 }
 
+// cell types, and bubble labels as dense cell indices, in dense order
+__global__ void k_export_types(Dev d, Geom g, uint8_t* dst) {
+  const long long n = (long long)g.nx * g.ny * g.nz;
+  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n;
+       u += (long long)gridDim.x * blockDim.x)
+    dst[u] = d.flags[u % g.nx + g.sx * (u / g.nx)] & F_TYPE;
+}
+__global__ void k_export_bubbles(Dev d, Geom g, int* dst) {
+  const long long n = (long long)g.nx * g.ny * g.nz;
+  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < n;
+       u += (long long)gridDim.x * blockDim.x) {
+    const int l = d.blab[u % g.nx + g.sx * (u / g.nx)];
+    // padded cell index -> dense index x + nx (y + ny z)
+    dst[u] = l >= 0 ? (l % g.sx) + g.nx * (l / g.sx) : l;
+  }
+}
+
 __global__ void k_set_trace(Ctrl* ctrl, int every) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     ctrl->trace_every = every;
@@ -270,7 +290,39 @@ fsl_status read_ctrl(fsl_handle* h, Ctrl* c) {
   return FSL_OK;
 }
 
+// Touch every page of an output buffer before the device writes it.  A large
+// array that the caller has just allocated has no pages yet, and a copy that
+// has to fault them in one after the other moves about 1 GB/s (the 134 MB fill
+// level of 256^3 cells: 119 ms); several host threads that write a byte per
+// page bring them in first, after which the copy runs at the link's rate.
+// The buffer is overwritten by the copy, so its content does not matter.
+void touch_pages(void* p, size_t bytes) {
+  constexpr size_t kPerThread = size_t(1) << 21;
+  if (!p || bytes < 2 * kPerThread) return;
+  const long ps = sysconf(_SC_PAGESIZE);
+  const size_t page = ps > 0 ? (size_t)ps : 4096;
+  size_t nt = std::min<size_t>(std::thread::hardware_concurrency(), 16);
+  nt = std::max<size_t>(1, std::min(nt, bytes / kPerThread));
+  volatile char* b = static_cast<volatile char*>(p);
+  const size_t part = (bytes / nt + page - 1) / page * page;
+  auto touch = [b, bytes, page, part](size_t t) {
+    const size_t end = std::min(bytes, (t + 1) * part);
+    for (size_t k = t * part; k < end; k += page) b[k] = 0;
+  };
+  std::vector<std::thread> th;
+  size_t started = 0;
+  try {
+    th.reserve(nt);
+    for (; started + 1 < nt; ++started) th.emplace_back(touch, started);
+  } catch (...) {
+    // no more threads: this one touches the rest
+  }
+  for (size_t t = started; t < nt; ++t) touch(t);
+  for (std::thread& t : th) t.join();
+}
+
 fsl_status copy_field(fsl_handle* h, const void* dev, size_t elem, void* host) {
+  touch_pages(host, (size_t)h->g.nx * elem * h->g.ny * h->g.nz);
   // padded rows (pitch sx) -> dense host rows (nx)
   FSL_CK(cudaMemcpy2DAsync(host, (size_t)h->g.nx * elem, dev, (size_t)h->g.sx * elem,
                            (size_t)h->g.nx * elem, (size_t)h->g.ny * h->g.nz,
@@ -523,24 +575,33 @@ fsl_status fsl_observe(fsl_handle* h, int what, void* host_out, size_t bytes) {
     case FSL_OBS_TRACE: {
       const int cnt = c.trace_count < kTraceCapacity ? c.trace_count : kTraceCapacity;
       if (bytes < (size_t)cnt * 3 * sizeof(double)) return FSL_ERR_ARG;
-      std::vector<double> ring((size_t)kTraceCapacity * 3);
-      FSL_CK(cudaMemcpyAsync(ring.data(), h->d.trace, ring.size() * sizeof(double),
-                             cudaMemcpyDeviceToHost, h->stream));
-      FSL_CK(cudaStreamSynchronize(h->stream));
-      const int first = c.trace_count - cnt;
+      // the records, oldest first: at most two stretches of the ring
+      const int first = (c.trace_count - cnt) % kTraceCapacity;
+      const int head = std::min(cnt, kTraceCapacity - first);
       double* o = static_cast<double*>(host_out);
-      for (int k = 0; k < cnt; ++k) {
-        const int slot = (first + k) % kTraceCapacity;
-        for (int j = 0; j < 3; ++j) o[3 * k + j] = ring[3 * slot + j];
-      }
+      if (head > 0)
+        FSL_CK(cudaMemcpyAsync(o, h->d.trace + 3 * (size_t)first, (size_t)head * 3 * sizeof(double),
+                               cudaMemcpyDeviceToHost, h->stream));
+      if (cnt > head)
+        FSL_CK(cudaMemcpyAsync(o + 3 * (size_t)head, h->d.trace, (size_t)(cnt - head) * 3 * sizeof(double),
+                               cudaMemcpyDeviceToHost, h->stream));
+      FSL_CK(cudaStreamSynchronize(h->stream));
       return FSL_OK;
     }
     case FSL_OBS_FIELD_PDF: {
       if (bytes < (size_t)q * n * sizeof(double)) return FSL_ERR_ARG;
       double* o = static_cast<double*>(host_out);
-      for (int i = 0; i < q; ++i) {
-        FSL_CK(h->L->export_pdf(h->d, h->g, h->p, cur, i, h->d.phinew, h->stream));
-        FSL_CK(cudaMemcpyAsync(o + (size_t)i * n, h->d.phinew, n * sizeof(double),
+      touch_pages(o, (size_t)q * n * sizeof(double));
+      // decoded into the other PDF buffer (the next step overwrites it), as many
+      // planes at a time as fit, and copied together
+      double* tmp = static_cast<double*>(h->d.pdf[cur ^ 1]);
+      const size_t room = (size_t)h->g.plane * q * storage_bytes(h->cfg.precision) / sizeof(double);
+      const int m = (int)std::min<size_t>(q, room / n);  // q / 4 planes or more
+      for (int i = 0; i < q; i += m) {
+        const int k = std::min(m, q - i);
+        for (int j = 0; j < k; ++j)
+          FSL_CK(h->L->export_pdf(h->d, h->g, h->p, cur, i + j, tmp + (size_t)j * n, h->stream));
+        FSL_CK(cudaMemcpyAsync(o + (size_t)i * n, tmp, (size_t)k * n * sizeof(double),
                                cudaMemcpyDeviceToHost, h->stream));
       }
       FSL_CK(cudaStreamSynchronize(h->stream));
@@ -548,10 +609,12 @@ fsl_status fsl_observe(fsl_handle* h, int what, void* host_out, size_t bytes) {
     }
     case FSL_OBS_FIELD_TYPES: {
       if (bytes < n) return FSL_ERR_ARG;
-      st = copy_field(h, h->d.flags, 1, host_out);
-      if (st != FSL_OK) return st;
-      unsigned char* o = static_cast<unsigned char*>(host_out);
-      for (size_t k = 0; k < n; ++k) o[k] &= F_TYPE;
+      touch_pages(host_out, n);
+      uint8_t* tmp = reinterpret_cast<uint8_t*>(h->d.phinew);  // scratch between steps
+      k_export_types<<<4 * 152, 256, 0, h->stream>>>(h->d, h->g, tmp);
+      FSL_CK(cudaGetLastError());
+      FSL_CK(cudaMemcpyAsync(host_out, tmp, n, cudaMemcpyDeviceToHost, h->stream));
+      FSL_CK(cudaStreamSynchronize(h->stream));
       return FSL_OK;
     }
     case FSL_OBS_FIELD_PHI:
@@ -570,11 +633,12 @@ fsl_status fsl_observe(fsl_handle* h, int what, void* host_out, size_t bytes) {
         for (size_t k = 0; k < n; ++k) o[k] = -1;
         return FSL_OK;
       }
-      fsl_status st2 = copy_field(h, h->d.blab, sizeof(int), host_out);
-      if (st2 != FSL_OK) return st2;
-      // padded cell index -> dense index x + nx (y + ny z)
-      for (size_t k = 0; k < n; ++k)
-        if (o[k] >= 0) o[k] = (o[k] % h->g.sx) + h->g.nx * (o[k] / h->g.sx);
+      touch_pages(host_out, n * sizeof(int));
+      int* tmp = reinterpret_cast<int*>(h->d.phinew);  // scratch between steps
+      k_export_bubbles<<<4 * 152, 256, 0, h->stream>>>(h->d, h->g, tmp);
+      FSL_CK(cudaGetLastError());
+      FSL_CK(cudaMemcpyAsync(host_out, tmp, n * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+      FSL_CK(cudaStreamSynchronize(h->stream));
       return FSL_OK;
     }
     case FSL_OBS_FIELD_PRESSURE: {
@@ -648,6 +712,7 @@ fsl_status fsl_save(fsl_handle* h, void* host_dst, size_t bytes) {
   std::vector<std::pair<char*, size_t>> parts;
   state_parts(h, c.step & 1, parts);
   char* o = static_cast<char*>(host_dst);
+  touch_pages(o, need);
   for (auto& pr : parts) {
     FSL_CK(cudaMemcpyAsync(o, pr.first, pr.second, cudaMemcpyDeviceToHost, h->stream));
     o += pr.second;
