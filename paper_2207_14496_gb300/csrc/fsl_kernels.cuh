@@ -19,16 +19,16 @@
 //                     fill level m/rho (Eq. nm-fslbm-mass), conversion marks
 //                     (threshold eps_phi) and warp-ballot compaction of the
 //                     to-liquid and to-gas cells;
-//   k_convert         one cooperative launch of five phases separated by
+//   k_convert         one cooperative launch of three phases separated by
 //                     grid-wide barriers (the batched path launches them one
 //                     by one):
-//     fill            commit fill levels; gas neighbours of filled cells become
+//     mark            commit fill levels; gas neighbours of filled cells become
 //                     new interface cells; to-gas neighbours are kept (filling
-//                     wins a conflict);
-//     empty           liquid neighbours of emptied cells become interface;
-//     finalise/share  type change, excess mass (Eq. nm-fslbm-excess-mass) and
-//                     its share per receiver, receiver compaction;
-//     refill          EQ, EQ+NEQ, GEQ, EXT, AVG refilling (Sec. 3.1);
+//                     wins a conflict); liquid neighbours of emptied cells
+//                     become interface;
+//     settle          type change, excess mass (Eq. nm-fslbm-excess-mass) and
+//                     its share per receiver, receiver compaction; EQ, EQ+NEQ,
+//                     GEQ, EXT, AVG refilling (Sec. 3.1) of the new cells;
 //     excess gather   receivers gather their shares in direction order;
 //   k_classify        Thuerey classes and curvature K = -div(n_hat) for the
 //                     next step, clean-up of the per-step marks, and the next
@@ -1552,22 +1552,34 @@ __global__ void __launch_bounds__(128, ST::kShift ? 5 : 1) kb_stream_collide_if(
 #define FSL_WARP_PER_ITEM(k, n)                                                     \
   for (unsigned k = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; k < (n);           \
        k += (gridDim.x * blockDim.x) >> 5)
+// the same with the items dealt out from the last warp of the grid on, so that
+// a second list of a phase keeps other warps busy than the first
+#define FSL_WARP_PER_ITEM_BACK(k, n)                                                \
+  for (unsigned k##_w = (gridDim.x * blockDim.x) >> 5,                              \
+                k = k##_w - 1u - ((threadIdx.x >> 5) * gridDim.x + blockIdx.x);     \
+       k < (n); k += k##_w)
 // one thread per item, spread over the blocks in the same way
 #define FSL_SPREAD_LOOP(k, n)                                                       \
   for (unsigned k = threadIdx.x * gridDim.x + blockIdx.x; k < (n);                  \
        k += gridDim.x * blockDim.x)
 
-template <int Q>
-__device__ __forceinline__ void fill_body(const Dev& d, const Geom& g) {
+// the fill levels computed by the interface pass become the cells' own
+__device__ __forceinline__ void commit_phi_body(const Dev& d) {
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
-  const unsigned nif = ctrl->n_if, nfill = ctrl->n_fill;
+  const unsigned nif = ctrl->n_if;
   const int* lif = list_if(d, ctrl->step);
-  // commit the fill levels computed by the stream-collide pass
   FSL_GRID_LOOP(k, nif) {
     const int c = lif[k];
     put_phi(d, c, d.phinew[c]);
   }
+}
+
+template <int Q>
+__device__ __forceinline__ void fill_body(const Dev& d, const Geom& g) {
+  Ctrl* ctrl = d.ctrl;
+  if (frozen(ctrl)) return;
+  const unsigned nfill = ctrl->n_fill;
   // gas neighbours of filled cells become new interface cells; a neighbour
   // about to empty is kept (filling wins)
   const int lane = threadIdx.x & 31;
@@ -1596,12 +1608,6 @@ __device__ __forceinline__ void fill_body(const Dev& d, const Geom& g) {
     warp_append(created, n, &ctrl->n_new, d.l_new);
   }
 }
-template <int Q>
-__global__ void __launch_bounds__(256) kb_fill(MemberTable t) {
-  FSL_MEMBER(t);
-  fill_body<Q>(d, g);
-}
-
 
 template <int Q, class ST>
 __device__ __forceinline__ void empty_body(const Dev& d, const Geom& g) {
@@ -1613,18 +1619,18 @@ __device__ __forceinline__ void empty_body(const Dev& d, const Geom& g) {
   const typename ST::T* A = (const typename ST::T*)d.pdf[cur];
   const unsigned ne = ctrl->n_empty;
   const int lane = threadIdx.x & 31;
-  FSL_WARP_PER_ITEM(k, ne) {
+  FSL_WARP_PER_ITEM_BACK(k, ne) {
     const int c = d.l_empty[k];
     int x, y, z;
     cell_xyz(g, c, x, y, z);
-    // the neighbour's flag byte is loaded together with the cell's own
     int n = -1;
     uint8_t fn = 0;
     if (lane >= 1 && lane < Q) {
       n = nb_at(g, x, y, z, rc(lane, 0), rc(lane, 1), rc(lane, 2));
       if (n >= 0) fn = d.flags[n];
     }
-    if (!(d.flags[c] & F_TO_GAS)) continue;  // kept by a filling neighbour (warp-uniform)
+    // kept by a filling neighbour (fill_body clears the mark meanwhile)
+    if (__any_sync(0xffffffffu, (fn & F_TO_LIQ) != 0)) continue;
     bool won = false;
     if (n >= 0 && (fn & F_TYPE) == T_LIQ) {
       // the liquid cell's density of this step, recomputed exactly as the
@@ -1648,21 +1654,16 @@ __device__ __forceinline__ void empty_body(const Dev& d, const Geom& g) {
     warp_append(won, n, &ctrl->n_l2i, d.l_l2i);
   }
 }
-template <int Q, class ST>
-__global__ void __launch_bounds__(256) kb_empty(MemberTable t) {
-  FSL_MEMBER(t);
-  empty_body<Q, ST>(d, g);
-}
-
 
 // Type of cell c once this step's conversions are applied: a cell marked to
 // fill becomes liquid, a cell still marked to empty becomes gas (every marked
 // cell is on the fill or the empty list, and the marks of earlier steps were
 // cleared by k_classify).  Beyond a wall: T_OBST.
-__device__ __forceinline__ int final_type(const uint8_t* flags, int c) {
-  if (c < 0) return T_OBST;
-  const uint8_t b = flags[c];
+__device__ __forceinline__ int final_type_of(uint8_t b) {
   return (b & F_TO_LIQ) ? T_LIQ : (b & F_TO_GAS) ? T_GAS : (b & F_TYPE);
+}
+__device__ __forceinline__ int final_type(const uint8_t* flags, int c) {
+  return c < 0 ? (int)T_OBST : final_type_of(flags[c]);
 }
 
 // Conversion of the filled and emptied cells with the share of their excess
@@ -1718,12 +1719,6 @@ __device__ __forceinline__ void finalise_share_body(const Dev& d, const Geom& g)
     }
   }
 }
-template <int Q>
-__global__ void __launch_bounds__(256) kb_finalise_share(MemberTable t) {
-  FSL_MEMBER(t);
-  finalise_share_body<Q>(d, g);
-}
-
 
 // ------------------------------------------------------------ normals
 // multiply-add with a weight that is a power of two: the product is exact, so
@@ -1740,8 +1735,9 @@ __device__ __forceinline__ double fma_pow2(double w, double d, double s) { retur
 // The 27 values are loaded once each, all in flight together (beyond a wall
 // the cell's own row or column stands in), and the flag bytes only where the
 // domain holds obstacle cells: a bit mask of the 27 cells decides each axis.
-template <class RC, class PT>
-__device__ __forceinline__ void normal_py(const Geom& g, const uint8_t* flags, const PT* phi, int x,
+// load(m): the fill level of cell m.
+template <class RC, class Load>
+__device__ __forceinline__ void normal_py(const Geom& g, const uint8_t* flags, Load&& load, int x,
                                           int y, int z, RC* n) {
   Nbr nb;
   nb.setup(g, x, y, z);
@@ -1756,7 +1752,7 @@ __device__ __forceinline__ void normal_py(const Geom& g, const uint8_t* flags, c
 #pragma unroll
   for (int k = 0; k < 27; ++k) {
     const int m = nb.in(k % 3 - 1, (k / 3) % 3 - 1, k / 9 - 1);
-    v[k] = (RC)phi[m];
+    v[k] = (RC)load(m);
     if (g.has_obst && (flags[m] & F_TYPE) == T_OBST) solid |= 1u << k;
   }
 #pragma unroll
@@ -1794,7 +1790,7 @@ template <class RC, class PT>
 __device__ __forceinline__ void unit_normal(const Geom& g, const uint8_t* flags, const PT* phi,
                                             int x, int y, int z, RC* nh) {
   RC n[3];
-  normal_py<RC>(g, flags, phi, x, y, z, n);
+  normal_py<RC>(g, flags, [phi](int m) { return phi[m]; }, x, y, z, n);
   const RC len = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
   const bool tiny = len < (RC)1e-12;
   const RC l = tiny ? (RC)1 : len;
@@ -1900,21 +1896,31 @@ __device__ inline void stored_moments_w(const typename ST::T* B, long long plane
   u[2] = jz / rho - (R)0.5 * PAR(R, p, g[2]);
 }
 
+// whether cell n is fluid after this step's conversions and was before
 __device__ __forceinline__ bool valid_src(const uint8_t* flags, int n) {
   if (n < 0) return false;
   const uint8_t f = flags[n];
-  return is_fluid(f & F_TYPE) && !(f & F_NEW);
+  return is_fluid(final_type_of(f)) && !(f & F_NEW);
 }
 
 // Refilling (Sec. 3.1), one warp per new interface cell: lane i examines the
 // neighbour x + c_i and writes the refilled f_i; sums over the valid
 // neighbours run in direction order (shuffled to every lane), so the FP64
-// result equals a sequential evaluation in that order.
+// result equals a sequential evaluation in that order.  What it reads of the
+// converted cells (type, fill level) it takes from their marks, so it does not
+// depend on finalise_share_body having run.
+// The neighbours' moments lie in shared memory for the sums: lanes 0..4 add up
+// one quantity each, one chain of q - 1 additions in place of five that every
+// lane ran on shuffled values (16 us for the four new cells of a step of a
+// 64x64 FP64 wave, now @@).
+constexpr int kMaxWarps = 16;  // warps of a block that runs refill_body
 template <int Q, class ST>
 __device__ __forceinline__ void refill_body(const Dev& d, const Geom& g, const Phys& p) {
   using T = typename ST::T;
   using R = typename ST::R;
   constexpr bool SH = ST::kShift;
+  __shared__ R moments[kMaxWarps][5][32];
+  auto& sm = moments[threadIdx.x >> 5];
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
   const int cur = ctrl->step & 1;
@@ -1924,7 +1930,7 @@ __device__ __forceinline__ void refill_body(const Dev& d, const Geom& g, const P
   const int lane = threadIdx.x & 31;
   const unsigned nn = ctrl->n_new;
   const int scheme = p.refill;
-  FSL_WARP_PER_ITEM(k, nn) {
+  FSL_WARP_PER_ITEM_BACK(k, nn) {
     const int c = d.l_new[k];
     int x, y, z;
     cell_xyz(g, c, x, y, z);
@@ -1941,19 +1947,24 @@ __device__ __forceinline__ void refill_body(const Dev& d, const Geom& g, const P
     const unsigned vmask = __ballot_sync(FULL, valid);
     const int count = __popc(vmask);
     // rho_bar, u_bar: plain means over the valid neighbours (R7)
-    R rsum = (R)0, dsum = (R)0, sx = (R)0, sy = (R)0, sz = (R)0;
-    for (int j = 1; j < Q; ++j) {
-      const R a = __shfl_sync(FULL, nr, j), b = __shfl_sync(FULL, ndr, j);
-      const R vx = __shfl_sync(FULL, nu[0], j), vy = __shfl_sync(FULL, nu[1], j),
-              vz = __shfl_sync(FULL, nu[2], j);
-      if ((vmask >> j) & 1u) {
-        rsum = rsum + a;
-        dsum = dsum + b;
-        sx = sx + vx;
-        sy = sy + vy;
-        sz = sz + vz;
+    __syncwarp();
+    sm[0][lane] = nr;
+    sm[1][lane] = ndr;
+    sm[2][lane] = nu[0];
+    sm[3][lane] = nu[1];
+    sm[4][lane] = nu[2];
+    __syncwarp();
+    R acc = (R)0;
+    if (lane < 5) {
+#pragma unroll 6
+      for (int j = 1; j < Q; ++j) {
+        const R v = sm[lane][j];
+        if ((vmask >> j) & 1u) acc = acc + v;
       }
     }
+    const R rsum = __shfl_sync(FULL, acc, 0), dsum = __shfl_sync(FULL, acc, 1);
+    const R sx = __shfl_sync(FULL, acc, 2), sy = __shfl_sync(FULL, acc, 3),
+            sz = __shfl_sync(FULL, acc, 4);
     const R cnt = (R)(count > 0 ? count : 1);
     const R rb = rsum / cnt, drb = dsum / cnt;
     const R ubx = sx / cnt, uby = sy / cnt, ubz = sz / cnt;
@@ -1961,7 +1972,15 @@ __device__ __forceinline__ void refill_body(const Dev& d, const Geom& g, const P
     int dn = -1;
     if (scheme == 1 || scheme == 3) {
       R n3[3];
-      normal_py<R>(g, d.flags, phi_work<R>(d), x, y, z, n3);
+      // fill levels after the conversions, from the marks: a converted cell's
+      // own entry may be written meanwhile (finalise_share_body)
+      const R* ph = phi_work<R>(d);
+      const uint8_t* fl = d.flags;
+      normal_py<R>(g, fl, [ph, fl](int m) {
+        const uint8_t b = fl[m];
+        const R v = ph[m];
+        return (b & F_TO_LIQ) ? (R)1 : (b & F_TO_GAS) ? (R)0 : v;
+      }, x, y, z, n3);
       R best = (R)0;
       for (int j = 1; j < Q; ++j) {
         if (!((vmask >> j) & 1u)) continue;
@@ -1994,11 +2013,8 @@ __device__ __forceinline__ void refill_body(const Dev& d, const Geom& g, const P
         }
       } else if (scheme == 2) {  // GEQ (R9: prefactor 1/(2 c_s^2 omega))
         R vel[7][3];
-        for (int j = 1; j <= 6; ++j) {
-          vel[j][0] = __shfl_sync(FULL, nu[0], j);
-          vel[j][1] = __shfl_sync(FULL, nu[1], j);
-          vel[j][2] = __shfl_sync(FULL, nu[2], j);
-        }
+        for (int j = 1; j <= 6; ++j)
+          for (int a = 0; a < 3; ++a) vel[j][a] = sm[2 + a][j];
         const R ub[3] = {ubx, uby, ubz};
         R du[3][3];
         for (int b = 0; b < 3; ++b) {
@@ -2051,20 +2067,17 @@ __device__ __forceinline__ void refill_body(const Dev& d, const Geom& g, const P
     }
     if (i < Q) ST::stw(B + i * P + c, out);
     // density of the refilled cell, summed in direction order
-    R r = (R)0;
-    for (int j = 0; j < Q; ++j) {
-      const R oj = __shfl_sync(FULL, out, j);
-      r = (j == 0) ? oj : r + oj;
+    __syncwarp();
+    sm[0][lane] = out;
+    __syncwarp();
+    if (lane == 0) {
+      R r = out;
+#pragma unroll 6
+      for (int j = 1; j < Q; ++j) r = r + sm[0][j];
+      d.rho[c] = SH ? 1.0 + (double)r : (double)r;
     }
-    if (lane == 0) d.rho[c] = SH ? 1.0 + (double)r : (double)r;
   }
 }
-template <int Q, class ST>
-__global__ void __launch_bounds__(128) kb_refill(MemberTable t) {
-  FSL_MEMBER(t);
-  refill_body<Q, ST>(d, g, p);
-}
-
 
 // ------------------------------------------------------------ excess mass
 // Each receiver gathers the shares of its converted neighbours, summed in
@@ -2111,14 +2124,19 @@ __global__ void __launch_bounds__(256) kb_excess_gather(MemberTable t) {
 
 
 // ------------------------------------------------------------ conversion phase
-// Fill, empty, finalise with excess share, refill and excess gather of one
-// step in one cooperative launch (all blocks resident).  Each phase reads what the
-// previous phases wrote anywhere in the domain, so a grid-wide barrier
+// The three phases of a step's conversions in one cooperative launch (all
+// blocks resident).  Each phase reads what the previous ones wrote anywhere
+// in the domain, so a grid-wide barrier
 // separates them: block arrivals are counted in ctrl->bar (phase k waits for
 // k * gridDim.x arrivals), the waits are bounded in time, and a block whose
 // wait gives up sets timeout bit 16 and leaves (the blocks still waiting then
 // give up in their turn).  The phases run the same bodies as the separate
 // kernels of the batched path, in the same order, so the results are the same.
+// The lists hold a few hundred to a few thousand cells, so a phase costs one
+// chain of dependent loads whatever it does: fill and empty share one (a cell
+// that stays because a neighbour fills sees that neighbour's mark itself), and
+// so do finalise and refill (types and fill levels after the conversions are
+// read from the marks).  Five phases took @@.
 constexpr unsigned long long kBarrierWaitNs = 200000000ull;  // 0.2 s
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
@@ -2129,19 +2147,21 @@ __device__ __forceinline__ bool grid_barrier(Ctrl* ctrl, unsigned target) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();  // this block's writes before its arrival
-    atomicAdd(&ctrl->bar, 1u);
+    // release: this block's writes before its arrival; acquire: the other
+    // blocks' writes before this block's reads
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&ctrl->bar) : "memory");
     int good = 1;
     const unsigned long long t0 = global_ns();
-    while (*(volatile unsigned*)&ctrl->bar < target) {
-      if (global_ns() - t0 > kBarrierWaitNs) {
+    for (unsigned spin = 1;; ++spin) {
+      unsigned seen;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&ctrl->bar) : "memory");
+      if (seen >= target) break;
+      if (spin % 64u == 0u && global_ns() - t0 > kBarrierWaitNs) {
         atomicOr(&ctrl->timeout, 16u);
         good = 0;
         break;
       }
-      __nanosleep(32);
     }
-    __threadfence();  // the other blocks' writes before this block's reads
     ok = good;
   }
   __syncthreads();
@@ -2162,20 +2182,36 @@ static __global__ void k_barrier_selftest(Dev d) {
   }
 }
 
+// One block per SM: an arrival at the barrier is an atomic on one address, and
+// with 608 blocks an empty phase cost 6-8 us, with 152 it costs 2.
+template <class ST>
+constexpr int convert_threads() { return ST::kShift ? 512 : 384; }
 template <int Q, class ST>
-__global__ void __launch_bounds__(256) k_convert(Dev d, Geom g, Phys p) {
+__global__ void __launch_bounds__(convert_threads<ST>(), 1) k_convert(Dev d, Geom g, Phys p) {
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
   const unsigned nb = gridDim.x;
   fill_body<Q>(d, g);
-  if (!grid_barrier(ctrl, nb)) return;
   empty_body<Q, ST>(d, g);
-  if (!grid_barrier(ctrl, 2 * nb)) return;
+  commit_phi_body(d);
+  if (!grid_barrier(ctrl, nb)) return;
   finalise_share_body<Q>(d, g);
-  if (!grid_barrier(ctrl, 3 * nb)) return;
   refill_body<Q, ST>(d, g, p);
-  if (!grid_barrier(ctrl, 4 * nb)) return;
+  if (!grid_barrier(ctrl, 2 * nb)) return;
   excess_gather_body<Q>(d, g);
+}
+template <int Q, class ST>
+__global__ void __launch_bounds__(256) kb_mark(MemberTable t) {
+  FSL_MEMBER(t);
+  fill_body<Q>(d, g);
+  empty_body<Q, ST>(d, g);
+  commit_phi_body(d);
+}
+template <int Q, class ST>
+__global__ void __launch_bounds__(256) kb_settle(MemberTable t) {
+  FSL_MEMBER(t);
+  finalise_share_body<Q>(d, g);
+  refill_body<Q, ST>(d, g, p);
 }
 
 
@@ -2791,26 +2827,26 @@ struct Kernels {
       }
     }
   }
-  // the conversion phase (k_convert), cooperative: at most four blocks per SM,
-  // as many as fit
+  // the conversion phase (k_convert), cooperative: one block per SM
   static cudaError_t convert(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
     static int grid = 0;
     if (grid == 0) {
       int per_sm = 0, dev = 0, sms = 0;
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_convert<Q, ST>, 256, 0);
+      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_convert<Q, ST>,
+                                                                    convert_threads<ST>(), 0);
       if (e != cudaSuccess) return e;
       e = cudaGetDevice(&dev);
       if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       if (e != cudaSuccess) return e;
       if (per_sm < 1) return cudaErrorLaunchOutOfResources;
-      grid = (per_sm < 4 ? per_sm : 4) * sms;
+      grid = sms;
     }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(convert_threads<ST>());
     cfg.dynamicSmemBytes = 0;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -3083,10 +3119,8 @@ struct Kernels {
       kb_stream_collide_if<Q, ST><<<dim3(16, m), 128, 0, s>>>(t);
       kb_tiles<kWarpTX><<<dim3((unsigned)bg.tiles, m), 256, 0, s>>>(t);
       kb_stream_collide_seg<Q, ST><<<dim3(32, m), 128, 0, s>>>(t);
-      kb_fill<Q><<<dim3(4, m), 256, 0, s>>>(t);
-      kb_empty<Q, ST><<<dim3(4, m), 256, 0, s>>>(t);
-      kb_finalise_share<Q><<<dim3(4, m), 256, 0, s>>>(t);
-      kb_refill<Q, ST><<<dim3(8, m), 128, 0, s>>>(t);
+      kb_mark<Q, ST><<<dim3(4, m), 256, 0, s>>>(t);
+      kb_settle<Q, ST><<<dim3(4, m), 256, 0, s>>>(t);
       kb_excess_gather<Q><<<dim3(4, m), 256, 0, s>>>(t);
       kb_classify<Q, ST><<<dim3(16, m), 128, 0, s>>>(t);
       kb_end_step<<<dim3(kEndBlocks, m), 256, 0, s>>>(t);
