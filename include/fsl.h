@@ -301,9 +301,9 @@ fsl_status fsl_total_mass_noalloc(const fsl_config* cfg, const void* d_pdf,
  * member by nsteps with one CUDA-graph launch per chunk of steps on the
  * batch's stream.  When every member stores 16- or 32-bit PDFs and none runs
  * the bubble model, each kernel of a step is launched once for all members
- * of a lattice and storage (up to 256 members per launch, one member per
+ * of a lattice and storage (up to 1024 members per launch, one member per
  * blockIdx.y; the member reads its pointers, geometry and parameters from a
- * record in its own workspace), so a step of the whole batch costs ten
+ * record in its own workspace), so a step of the whole batch costs eight
  * launches; otherwise each member's kernels form an independent branch
  * (a child graph per member, no edges between members).  Either way the GPU
  * runs the domains side by side instead of one after another.

@@ -1530,10 +1530,233 @@ __device__ __forceinline__ void stream_collide_if_body(const Dev& d, const Geom&
   }
   if (bad) atomicCAS(&ctrl->unstable_step, -1, ctrl->step + 1);
 }
+// The same pass for the single domains of D3Q19: one thread per cell, its q own
+// values, pulled values and neighbour fill
+// levels in a column of shared memory.  The values of all directions are
+// loaded together (registers could hold a third of them), and the boundary
+// condition and the flux run over the opposite pairs in a rolled loop: the
+// former fully unrolled code of 3,500 instructions was run through once per
+// warp and waited on instruction fetch and on one pair's loads after the
+// other (87 cells of a 64x64 FP64 wave: 33 -> 29 us, 4,300 of a 512x256x16 FP32
+// dam break: 21 -> 14, 160,000 of a bubbly channel: 78 -> 68).  Not for D3Q27,
+// whose columns take the shared memory that the gathers need as L1 (83,000
+// cells of a 256^3 FP16 drop impact: 62 -> 98 us, 160^3 FP64: 94 -> 185), nor
+// for batches (many blocks of few cells: 49 -> 61 us).
+template <int Q, class R>
+struct IfColumn {
+  static constexpr int threads = 128;
+  // direction i (1 .. Q - 1) in row i - 1
+  R own[Q - 1][threads];  // stored values of the cell
+  R fin[Q - 1][threads];  // pulled values
+  R phi[Q - 1][threads];  // fill level of the source cell of direction i
+  uint8_t fb[Q - 1][threads];  // its flag byte; T_OBST where the source is solid
+};
+
+template <int Q, class ST, int AX>
+__device__ __forceinline__ void stream_collide_col_body(const Dev& d, const Geom& g, const Phys& p) {
+  using T = typename ST::T;
+  using R = typename ST::R;
+  using Col = IfColumn<Q, R>;
+  constexpr bool SH = ST::kShift;
+  extern __shared__ __align__(16) unsigned char if_smem[];
+  Col& col = *reinterpret_cast<Col*>(if_smem);
+  const int tid = threadIdx.x;
+  Ctrl* ctrl = d.ctrl;
+  if (frozen(ctrl)) return;
+  const int cur = ctrl->step & 1;
+  const T* __restrict__ A = (const T*)d.pdf[cur];
+  T* __restrict__ B = (T*)d.pdf[cur ^ 1];
+  const long long P = g.plane;
+  const unsigned nif = ctrl->n_if;
+  const int* lif = list_if(d, ctrl->step);
+  bool bad = false;
+  // 32 consecutive list entries per warp; the warps of a list that does not
+  // fill the blocks go to one block (one SM) after the other
+  const unsigned nw = blockDim.x >> 5, warp = tid >> 5;
+  const unsigned w0 = nif <= 32u * gridDim.x ? warp * gridDim.x + blockIdx.x : blockIdx.x * nw + warp;
+#pragma unroll 1
+  for (unsigned base = 32u * w0; base < nif; base += 32u * nw * gridDim.x) {
+    const unsigned k = base + (tid & 31);
+    const bool ok = k < nif;
+    bool to_liq = false, to_gas = false;
+    const int c = ok ? lif[k] : 0;
+    if (ok) {
+    int x, y, z;
+    cell_xyz(g, c, x, y, z);
+    const uint8_t fl = d.flags[c];
+    // directions whose source lies beyond a wall; there the coordinate that
+    // crosses it is the cell's own (the mirror image across a free-slip wall)
+    Nbr nb;
+    nb.setup(g, x, y, z);
+    unsigned cross = 0u;
+    if (nb.X[0] < 0) { cross |= dirs_with<Q>(0, 1); nb.X[0] = x; }
+    if (nb.X[2] < 0) { cross |= dirs_with<Q>(0, -1); nb.X[2] = x; }
+    if (nb.Y[0] < 0) { cross |= dirs_with<Q>(1, 1); nb.Y[0] = y; }
+    if (nb.Y[2] < 0) { cross |= dirs_with<Q>(1, -1); nb.Y[2] = y; }
+    if (nb.Z[0] < 0) { cross |= dirs_with<Q>(2, 1); nb.Z[0] = z; }
+    if (nb.Z[2] < 0) { cross |= dirs_with<Q>(2, -1); nb.Z[2] = z; }
+    const R* __restrict__ phi = phi_work<R>(d);
+    R own[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) own[i] = ST::ldw(A + i * P + c);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const int n = nb.in(-dir_c(i, 0), -dir_c(i, 1), -dir_c(i, 2));
+      const uint8_t b = d.flags[n];
+      col.fin[i - 1][tid] = ST::ldw(A + i * P + n);
+      col.phi[i - 1][tid] = phi[n];
+      col.fb[i - 1][tid] = (cross >> i) & 1u ? (uint8_t)T_OBST : b;
+    }
+    if (cross && g.free_slip) {
+      // across free-slip walls the value comes in the mirrored direction
+#pragma unroll 1
+      for (unsigned m = cross; m; m &= m - 1) {
+        const int i = __ffs(m) - 1;
+        const int cx = rc(i, 0), cy = rc(i, 1), cz = rc(i, 2);
+        const int walls = ((x - cx < 0 || x - cx >= g.nx) && !g.periodic[0] ? 1 : 0) |
+                          ((y - cy < 0 || y - cy >= g.ny) && !g.periodic[1] ? 2 : 0) |
+                          ((z - cz < 0 || z - cz >= g.nz) && !g.periodic[2] ? 4 : 0);
+        if ((walls & g.free_slip) != walls) continue;  // also a no-slip wall: bounced back
+        const int n = (cx == 0 ? x : cx > 0 ? nb.X[0] : nb.X[2]) +
+                      g.sx * ((cy == 0 ? y : cy > 0 ? nb.Y[0] : nb.Y[2]) +
+                              g.ny * (cz == 0 ? z : cz > 0 ? nb.Z[0] : nb.Z[2]));
+        col.fin[i - 1][tid] = ST::ldw(A + mirror_dir<Q>(i, walls) * P + n);
+        col.fb[i - 1][tid] = d.flags[n];
+      }
+    }
+    // stored post-collision moments at t: u = sum c f* / rho - g / 2
+    R rt, drt, jx, jy, jz;
+    density<Q, SH, R>(own, rt, drt);
+    momentum<Q, R>(own, jx, jy, jz);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) col.own[i - 1][tid] = own[i];
+    const R utx = jx / rt - (R)0.5 * PAR(R, p, g[0]);
+    const R uty = jy / rt - (R)0.5 * PAR(R, p, g[1]);
+    const R utz = jz / rt - (R)0.5 * PAR(R, p, g[2]);
+    const R utsq = utx * utx + uty * uty + utz * utz;
+    // Eq. nm-fslbm-pressure-gas: volume pressure (per bubble with the bubble
+    // model, Eq. nm-fslbm-pressure-volume) and Laplace pressure
+    int bub = -1;
+    if (g.bubbles) bub = d.blab[c];
+    const double pv = bub >= 0 ? d.bp[bub] : p.p_v;
+    const double pg = (p.options & 8u) ? pv - 2.0 * p.sigma * d.kappa[c]
+                                       : pv + p.sigma * d.kappa[c];
+    const R rg = (R)(3.0 * pg);  // rho_G = p_G / c_s^2
+    const R drg = (R)(3.0 * pg - 1.0);
+    // Eq. nm-fslbm-mass-flux over i = 1..Q-1 (gas and walls carry none), in
+    // the working precision (FP64 in the FP64 path)
+    const R phx = phi[c];
+    const int clsx = fl & (F_NF | F_NE);
+    const bool thurey = !(p.options & 1u);
+    R dm = (R)0;
+    bool dm_has = false;
+    // one flux term: t, b, ph of the cell that exchanges PDFs with x along
+    // c_i (the source of the incoming f_io), in = what arrives from it, out =
+    // f*_i(x)
+    auto flux = [&](uint8_t b, R ph, R in, R out, R w) {
+      const int t = b & F_TYPE;
+      if (t != T_LIQ && t != T_IF) return;
+      R dd;
+      const R both = in - out;
+      if (t == T_LIQ) {
+        dd = both;
+      } else {
+        const int clsn = b & (F_NF | F_NE);
+        const R f_in = SH ? in + w : in;
+        const R f_out = SH ? out + w : out;
+        R br;
+        if (!thurey) br = both;
+        else if (clsx == 0) br = (clsn == F_NF) ? f_in : (clsn == F_NE) ? -f_out : both;
+        else if (clsx == F_NF) br = (clsn == F_NF) ? both : -f_out;
+        else br = (clsn == F_NE) ? both : f_in;
+        dd = (R)0.5 * (phx + ph) * br;
+      }
+      dm = dm_has ? dm + dd : dd;
+      dm_has = true;
+    };
+    // opposite pairs (i, i + 1) = (1, 2), (3, 4), ...: the pulled values, then
+    // the pair's two flux terms, so that the sum runs over i = 1, 2, 3, ...
+#pragma unroll 1
+    for (int q = 0; q < (Q - 1) / 2; ++q) {
+      const int i = 2 * q + 1;
+      const R w = pair_weight<Q, R>(q);
+      const uint8_t b0 = col.fb[i - 1][tid], b1 = col.fb[i][tid];
+      const int t0 = b0 & F_TYPE, t1 = b1 & F_TYPE;
+      const R o0 = col.own[i - 1][tid], o1 = col.own[i][tid];
+      R f0 = col.fin[i - 1][tid], f1 = col.fin[i][tid];  // neighbour or mirror image
+      if (t0 == T_OBST) f0 = o1;                         // halfway bounce-back
+      if (t1 == T_OBST) f1 = o0;
+      if (t0 == T_GAS || t1 == T_GAS) {
+        // anti-bounce-back from gas (Eq. nm-fslbm-boundary-condition): the sum
+        // of the pair's equilibria at the gas density
+        const int cx = rc(i, 0), cy = rc(i, 1), cz = rc(i, 2);
+        const R ax = cx == 0 ? (R)0 : cx > 0 ? utx : -utx;
+        const R ay = cy == 0 ? (R)0 : cy > 0 ? uty : -uty;
+        const R az = cz == 0 ? (R)0 : cz > 0 ? utz : -utz;
+        const R cu = (ax + ay) + az;
+        R fa, fo;
+        if constexpr (SH) {
+          const R c3 = (R)3 * cu, cc = (R)4.5 * cu * cu, h = (R)1.5 * utsq;
+          fa = w * (drg + rg * (c3 + cc - h));
+          fo = w * (drg + rg * (-c3 + cc - h));
+        } else {
+          const R c3 = (R)3 * cu, cc = (R)4.5 * cu * cu, h = (R)1.5 * utsq;
+          fa = w * rg * ((R)1 + c3 + cc - h);
+          fo = w * rg * ((R)1 - c3 + cc - h);
+        }
+        const R both = fa + fo;
+        if (t0 == T_GAS) f0 = both - o1;
+        if (t1 == T_GAS) f1 = both - o0;
+      }
+      col.fin[i - 1][tid] = f0;
+      col.fin[i][tid] = f1;
+      flux(b1, col.phi[i][tid], f1, o0, w);
+      flux(b0, col.phi[i - 1][tid], f0, o1, w);
+    }
+    const double m_new = dm_has ? d.mass[c] + (double)dm : d.mass[c];
+    R fin[Q], fout[Q], rho;
+    fin[0] = own[0];
+#pragma unroll
+    for (int i = 1; i < Q; ++i) fin[i] = col.fin[i - 1][tid];
+    R usq;
+    if constexpr (SH) {
+      // 16/32-bit path: the regrouped pair collision of the bulk kernels, on
+      // unscaled offsets (scale 1); rho summed in the same pair order
+      R drho;
+      density<Q, SH, R>(fin, rho, drho);
+      const bool tr = p.trt != 0;
+      usq = collide_v<Q, float>(fin, fout, p.f.lam_e, tr ? p.f.lam_o : p.f.omega, p.f.pre_e,
+                                tr ? p.f.pre_o : p.f.pre_e, p.f.g[0], p.f.g[1], p.f.g[2], 1.0f,
+                                LesLp::of(p));
+    } else {
+      usq = collide64<Q, AX>(fin, fout, p, rho);
+    }
+    if (!(usq < (R)(1.0 / 3.0))) bad = true;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) ST::stw(B + i * P + c, fout[i]);
+    const double rd = (double)rho;
+    const double ph = m_new / rd;  // Eq. nm-fslbm-mass
+    d.mass[c] = m_new;
+    d.rho[c] = rd;
+    d.phinew[c] = ph;
+    if (ph > p.thr_hi) {
+      d.flags[c] = fl | F_TO_LIQ;
+      to_liq = true;
+    } else if (ph < p.thr_lo) {
+      d.flags[c] = fl | F_TO_GAS;
+      to_gas = true;
+    }
+    }
+    warp_append(to_liq, c, &ctrl->n_fill, d.l_fill);
+    warp_append(to_gas, c, &ctrl->n_empty, d.l_empty);
+  }
+  if (bad) atomicCAS(&ctrl->unstable_step, -1, ctrl->step + 1);
+}
 // AX: force axis of the FP64 collision (unused by the 16/32-bit storages)
 template <int Q, class ST, int AX>
 __global__ void __launch_bounds__(128, ST::kShift ? 5 : 1) k_stream_collide_if(Dev d, Geom g, Phys p) {
-  stream_collide_if_body<Q, ST, AX>(d, g, p);
+  if constexpr (Q == 19) stream_collide_col_body<Q, ST, AX>(d, g, p);
+  else stream_collide_if_body<Q, ST, AX>(d, g, p);
 }
 template <int Q, class ST>
 __global__ void __launch_bounds__(128, ST::kShift ? 5 : 1) kb_stream_collide_if(MemberTable t) {
@@ -2796,7 +3019,8 @@ struct Kernels {
       if (e == cudaSuccess) e = cudaStreamWaitEvent(aux.side, aux.fork, 0);
       if (e != cudaSuccess) return e;
     }
-    interface_pass(d, g, p, si);
+    e = interface_pass(d, g, p, si);
+    if (e != cudaSuccess) return e;
     if (aux.side) {
       e = cudaEventRecord(aux.join, aux.side);
       if (e != cudaSuccess) return e;
@@ -2815,15 +3039,25 @@ struct Kernels {
     k_end_step<<<kEndBlocks, 256, 0, s>>>(d, g);
     return cudaGetLastError();
   }
-  static void interface_pass(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
+  static constexpr size_t kIfSmem = Q == 19 ? sizeof(IfColumn<Q, typename ST::R>) : 0;
+  template <int AX>
+  static cudaError_t interface_pass_as(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
+    static const cudaError_t e =
+        cudaFuncSetAttribute(k_stream_collide_if<Q, ST, AX>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIfSmem);
+    if (e != cudaSuccess) return e;
+    k_stream_collide_if<Q, ST, AX><<<kCellListBlocks, 128, kIfSmem, s>>>(d, g, p);
+    return cudaGetLastError();
+  }
+  static cudaError_t interface_pass(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
     if constexpr (ST::kShift) {
-      k_stream_collide_if<Q, ST, 3><<<kCellListBlocks, 128, 0, s>>>(d, g, p);
+      return interface_pass_as<3>(d, g, p, s);
     } else {
       switch (force_axis(p)) {
-        case 0: k_stream_collide_if<Q, ST, 0><<<kCellListBlocks, 128, 0, s>>>(d, g, p); break;
-        case 1: k_stream_collide_if<Q, ST, 1><<<kCellListBlocks, 128, 0, s>>>(d, g, p); break;
-        case 2: k_stream_collide_if<Q, ST, 2><<<kCellListBlocks, 128, 0, s>>>(d, g, p); break;
-        default: k_stream_collide_if<Q, ST, 3><<<kCellListBlocks, 128, 0, s>>>(d, g, p);
+        case 0: return interface_pass_as<0>(d, g, p, s);
+        case 1: return interface_pass_as<1>(d, g, p, s);
+        case 2: return interface_pass_as<2>(d, g, p, s);
+        default: return interface_pass_as<3>(d, g, p, s);
       }
     }
   }

@@ -50,6 +50,24 @@ static __constant__ double kW27[27] = {
     wgt<27>(7),  wgt<27>(8),  wgt<27>(9),  wgt<27>(10), wgt<27>(11), wgt<27>(12), wgt<27>(13),
     wgt<27>(14), wgt<27>(15), wgt<27>(16), wgt<27>(17), wgt<27>(18), wgt<27>(19), wgt<27>(20),
     wgt<27>(21), wgt<27>(22), wgt<27>(23), wgt<27>(24), wgt<27>(25), wgt<27>(26)};
+// the weights of the odd directions 1, 3, ... (opposite pairs share one) in the
+// arithmetic type R
+template <int Q, class R>
+struct PairWeights {
+  R w[(Q - 1) / 2];
+  constexpr PairWeights() : w() {
+    for (int k = 0; k < (Q - 1) / 2; ++k) w[k] = (R)wgt<Q>(2 * k + 1);
+  }
+};
+static __constant__ PairWeights<19, double> kPairW19d;
+static __constant__ PairWeights<27, double> kPairW27d;
+static __constant__ PairWeights<19, float> kPairW19f;
+static __constant__ PairWeights<27, float> kPairW27f;
+template <int Q, class R>
+__device__ __forceinline__ R pair_weight(int k) {
+  if constexpr (sizeof(R) == 8) return Q == 19 ? kPairW19d.w[k] : kPairW27d.w[k];
+  else return Q == 19 ? kPairW19f.w[k] : kPairW27f.w[k];
+}
 __device__ __forceinline__ int rc(int i, int a) { return kDirC[i][a]; }
 template <int Q>
 __device__ __forceinline__ double rw(int i) {
