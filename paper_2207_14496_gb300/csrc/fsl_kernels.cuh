@@ -2714,74 +2714,105 @@ __device__ inline int block_max(int v, int* sh) {
   return r;
 }
 
+// Sum of v and maxima of a and b over a block of 256 threads, in the tree of
+// block_sum and block_max (thread t takes t + 128, t + 64, ..., t + 1), the
+// three together and the last five levels by shuffles; in thread 0.
+__device__ __forceinline__ void block_reduce3(double& v, int& a, int& b, double* shd, int* sha,
+                                              int* shb) {
+  const int t = threadIdx.x;
+  shd[t] = v;
+  sha[t] = a;
+  shb[t] = b;
+  __syncthreads();
+#pragma unroll
+  for (int s = 128; s >= 32; s >>= 1) {
+    if (t < s) {
+      shd[t] = v = v + shd[t + s];
+      sha[t] = a = max(a, sha[t + s]);
+      shb[t] = b = max(b, shb[t + s]);
+    }
+    __syncthreads();
+  }
+  if (t < 32) {
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+      v = v + __shfl_down_sync(0xffffffffu, v, s);
+      a = max(a, __shfl_down_sync(0xffffffffu, a, s));
+      b = max(b, __shfl_down_sync(0xffffffffu, b, s));
+    }
+  }
+}
+
 // End of step: optional trace record, counters for the next step, step++.
-// The trace reductions are split over kEndBlocks blocks (fixed partition,
-// fixed tree order); the last block to finish combines the partials in block
-// order and advances the counters.
+// The trace reductions are split into kEndBlocks parts (fixed partition,
+// fixed tree order), whatever the number of blocks that work on them; the
+// last block to finish combines the partials in part order and advances the
+// counters.  A handle that never traces needs none of that: block 0 alone
+// advances the counters.
 constexpr int kEndBlocks = 64;
 __device__ __forceinline__ void end_step_body(const Dev& d, const Geom& g) {
   __shared__ double shd[256];
-  __shared__ int shi[256];
+  __shared__ int sha[256], shb[256];
   __shared__ bool last;
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
   const int every = ctrl->trace_every;
+  if (every == 0 && blockIdx.x != 0) return;
   const bool tracing = every > 0 && ((ctrl->step + 1) % every) == 0;
   double* part = d.red;                         // kEndBlocks column partials
   int* ipart = reinterpret_cast<int*>(d.red + kEndBlocks);  // 2 x kEndBlocks maxima
   if (tracing) {
     const int ncol = g.ny * g.nz;
-    const int chunk = (ncol + gridDim.x - 1) / gridDim.x;
-    const int k0 = blockIdx.x * chunk, k1 = min(ncol, k0 + chunk);
-    double s = 0.0;
-    int hbest = -1;
-    for (int k = k0 + threadIdx.x; k < k1; k += 256) {
-      const long long cidx = (long long)g.sx * k;   // cell (0, j, kz), k = j + ny kz
-      s += d.phi[cidx];
-      if ((d.flags[cidx] & F_TYPE) == T_IF) hbest = max(hbest, k % g.ny);
-    }
-    const double bs = block_sum<256>(s, shd);
-    const int bh = block_max<256>(hbest, shi);
-    // front: cells (i, 0, kz)
+    const int chunk = (ncol + kEndBlocks - 1) / kEndBlocks;
     const int nrow = g.nx * g.nz;
-    const int rchunk = (nrow + gridDim.x - 1) / gridDim.x;
-    const int r0 = blockIdx.x * rchunk, r1 = min(nrow, r0 + rchunk);
-    int fbest = -1;
-    for (int k = r0 + threadIdx.x; k < r1; k += 256) {
-      const int i = k % g.nx, kz = k / g.nx;
-      if ((d.flags[i + (long long)g.sx * g.ny * kz] & F_TYPE) == T_IF) fbest = max(fbest, i);
-    }
-    const int bf = block_max<256>(fbest, shi);
-    if (threadIdx.x == 0) {
-      part[blockIdx.x] = bs;
-      ipart[blockIdx.x] = bf;
-      ipart[kEndBlocks + blockIdx.x] = bh;
+    const int rchunk = (nrow + kEndBlocks - 1) / kEndBlocks;
+    for (int vb = blockIdx.x; vb < kEndBlocks; vb += gridDim.x) {
+      const int k0 = vb * chunk, k1 = min(ncol, k0 + chunk);
+      double s = 0.0;
+      int hbest = -1;
+      for (int k = k0 + threadIdx.x; k < k1; k += 256) {
+        const long long cidx = (long long)g.sx * k;   // cell (0, j, kz), k = j + ny kz
+        s += d.phi[cidx];
+        if ((d.flags[cidx] & F_TYPE) == T_IF) hbest = max(hbest, k % g.ny);
+      }
+      // front: cells (i, 0, kz)
+      const int r0 = vb * rchunk, r1 = min(nrow, r0 + rchunk);
+      int fbest = -1;
+      for (int k = r0 + threadIdx.x; k < r1; k += 256) {
+        const int i = k % g.nx, kz = k / g.nx;
+        if ((d.flags[i + (long long)g.sx * g.ny * kz] & F_TYPE) == T_IF) fbest = max(fbest, i);
+      }
+      block_reduce3(s, fbest, hbest, shd, sha, shb);
+      if (threadIdx.x == 0) {
+        part[vb] = s;
+        ipart[vb] = fbest;
+        ipart[kEndBlocks + vb] = hbest;
+      }
     }
   }
-  __threadfence();
-  if (threadIdx.x == 0) last = atomicAdd(&ctrl->end_blocks, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  if (tracing) {
-    const bool in = (int)threadIdx.x < (int)gridDim.x;
-    const double cp = in ? *(volatile double*)&part[threadIdx.x] : 0.0;
-    const int fp = in ? *(volatile int*)&ipart[threadIdx.x] : -1;
-    const int hp = in ? *(volatile int*)&ipart[kEndBlocks + threadIdx.x] : -1;
-    const double col_all = block_sum<256>(cp, shd);
-    const int front_all = block_max<256>(fp, shi);
-    const int height_all = block_max<256>(hp, shi);
-    if (threadIdx.x == 0) {
-      shd[0] = col_all;
-      shi[0] = front_all;
-      shi[1] = height_all;
-    }
+  if (every > 0) {
+    __threadfence();
+    if (threadIdx.x == 0) last = atomicAdd(&ctrl->end_blocks, 1u) == gridDim.x - 1;
     __syncthreads();
+    if (!last) return;
+    __threadfence();
+  }
+  if (tracing) {
+    const bool in = (int)threadIdx.x < kEndBlocks;
+    double cp = in ? *(volatile double*)&part[threadIdx.x] : 0.0;
+    int fp = in ? *(volatile int*)&ipart[threadIdx.x] : -1;
+    int hp = in ? *(volatile int*)&ipart[kEndBlocks + threadIdx.x] : -1;
+    block_reduce3(cp, fp, hp, shd, sha, shb);
+    if (threadIdx.x == 0) {
+      shd[0] = cp;
+      sha[0] = fp;
+      shb[0] = hp;
+    }
   }
   if (threadIdx.x == 0) {
     if (tracing) {
       const double col = shd[0];
-      const int front = shi[0], height = shi[1];
+      const int front = sha[0], height = shb[0];
       const int slot = ctrl->trace_count % kTraceCapacity;
       d.trace[3 * slot + 0] = col / (double)g.nz;
       d.trace[3 * slot + 1] = (double)(front + 1);
@@ -3356,8 +3387,8 @@ struct Kernels {
       kb_mark<Q, ST><<<dim3(4, m), 256, 0, s>>>(t);
       kb_settle<Q, ST><<<dim3(4, m), 256, 0, s>>>(t);
       kb_excess_gather<Q><<<dim3(4, m), 256, 0, s>>>(t);
-      kb_classify<Q, ST><<<dim3(16, m), 128, 0, s>>>(t);
-      kb_end_step<<<dim3(kEndBlocks, m), 256, 0, s>>>(t);
+      kb_classify<Q, ST><<<dim3(8, m), 128, 0, s>>>(t);
+      kb_end_step<<<dim3(4, m), 256, 0, s>>>(t);
       return cudaGetLastError();
     } else {
       (void)t; (void)n; (void)bg; (void)s;
