@@ -2633,48 +2633,58 @@ static __global__ void k_list_interface(Dev d, Geom g) {
 // consecutive cells in order with one atomic; n_if_next and end_blocks, zero
 // between steps, count, and the last block clears them again (the count is the
 // n_if that the step already has).
-constexpr int kSortCells = 256 * 64;
+constexpr int kSortRounds = 4;  // 16 cells per thread and round
+constexpr int kSortCells = 256 * 16 * kSortRounds;
 __device__ __forceinline__ void sort_interface_body(const Dev& d, const Geom& g) {
-  __shared__ unsigned warp_n[8];
+  __shared__ unsigned warp_n[kSortRounds][8];
   __shared__ unsigned base;
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
-  const long long c0 = blockIdx.x * (long long)kSortCells + 64 * threadIdx.x;
+  const long long c0 = blockIdx.x * (long long)kSortCells + 16 * threadIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long mask = 0;  // interface cells among the thread's 64
-  if (c0 < g.cells) {
-    // rows are padded to multiples of 32 cells: two 16-byte words at a time
+  unsigned mask[kSortRounds], before[kSortRounds];  // interface cells; those of lower lanes
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (c0 + 16 * q >= g.cells) break;
-      const uint4 v = *reinterpret_cast<const uint4*>(d.flags + c0 + 16 * q);
+  for (int q = 0; q < kSortRounds; ++q) {
+    const long long c = c0 + 4096 * q;  // (rows are padded to multiples of 32 cells)
+    mask[q] = 0u;
+    if (c < g.cells) {
+      const uint4 v = *reinterpret_cast<const uint4*>(d.flags + c);
       const unsigned u[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int h = 0; h < 16; ++h)
-        if (((u[h / 4] >> (8 * (h % 4))) & F_TYPE) == T_IF) mask |= 1ull << (16 * q + h);
+        if (((u[h / 4] >> (8 * (h % 4))) & F_TYPE) == T_IF) mask[q] |= 1u << h;
     }
   }
-  const unsigned n = (unsigned)__popcll(mask);
-  unsigned before = n;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned t = __shfl_up_sync(0xffffffffu, before, o);
-    if (lane >= o) before += t;
+  for (int q = 0; q < kSortRounds; ++q) {
+    const unsigned n = (unsigned)__popc(mask[q]);
+    unsigned t = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned k = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += k;
+    }
+    before[q] = t - n;
+    if (lane == 31) warp_n[q][warp] = t;
   }
-  if (lane == 31) warp_n[warp] = before;
   __syncthreads();
   if (threadIdx.x == 0) {
     unsigned t = 0;
-    for (int w = 0; w < 8; ++w) {
-      const unsigned k = warp_n[w];
-      warp_n[w] = t;
-      t += k;
-    }
+    for (int q = 0; q < kSortRounds; ++q)
+      for (int w = 0; w < 8; ++w) {
+        const unsigned k = warp_n[q][w];
+        warp_n[q][w] = t;
+        t += k;
+      }
     base = t ? atomicAdd(&ctrl->n_if_next, t) : 0u;
   }
   __syncthreads();
-  int* out = list_if(d, ctrl->step) + base + warp_n[warp] + before - n;
-  for (; mask; mask &= mask - 1) *out++ = (int)(c0 + __ffsll(mask) - 1);
+  int* list = list_if(d, ctrl->step);
+#pragma unroll
+  for (int q = 0; q < kSortRounds; ++q) {
+    int* out = list + base + warp_n[q][warp] + before[q];
+    for (unsigned m = mask[q]; m; m &= m - 1) *out++ = (int)(c0 + 4096 * q + __ffs(m) - 1);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
