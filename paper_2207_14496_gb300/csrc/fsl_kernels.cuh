@@ -1347,15 +1347,21 @@ namespace fsl {
 // ------------------------------------------------------------ stream-collide
 // FP64 pass over all cells: liquid cells stream and collide here (interface cells
 // are handled by k_stream_collide_if from the step's interface list).
-template <int Q, int AX>
-__global__ void __launch_bounds__(128) k_stream_collide(Dev d, Geom g, Phys p) {
+// One warp per block, 32 cells of a row: blocks of 128 cells left warps of a
+// row's last block empty (three of eight for 160 cells) and dealt small domains
+// out unevenly.  At least MINB warps fit an SM, which keeps the FP64 pipes fed
+// through the loads and leaves room for the interface pass beside it.
+// (400x400 FP64 wave, step: 113 us before, 101 so; 160^3 drop impact: 2,027 us,
+// 1,981 so.)
+template <int Q, int AX, int MINB>
+__global__ void __launch_bounds__(32, MINB) k_stream_collide(Dev d, Geom g, Phys p) {
   using ST = SF64;
   using T = double;
   using R = double;
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
   const int cur = ctrl->step & 1;  // pdf[step & 1] holds f*(t)
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
   const T* __restrict__ A = (const T*)d.pdf[cur];
   T* __restrict__ B = (T*)d.pdf[cur ^ 1];
   const long long P = g.plane;
@@ -3259,6 +3265,16 @@ struct Kernels {
     }
     return cudaSuccess;
   }
+  template <int MINB>
+  static void bulk_fp64(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
+    const dim3 n((g.nx + 31) / 32, g.ny, g.nz);
+    switch (force_axis(p)) {
+      case 0: k_stream_collide<Q, 0, MINB><<<n, 32, 0, s>>>(d, g, p); break;
+      case 1: k_stream_collide<Q, 1, MINB><<<n, 32, 0, s>>>(d, g, p); break;
+      case 2: k_stream_collide<Q, 2, MINB><<<n, 32, 0, s>>>(d, g, p); break;
+      default: k_stream_collide<Q, 3, MINB><<<n, 32, 0, s>>>(d, g, p);
+    }
+  }
   static cudaError_t stream_collide(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
     if constexpr (ST::kShift) {
       const int v = variant_of(g);
@@ -3364,13 +3380,9 @@ struct Kernels {
           k_stream_collide_lp<Q, ST, 128, 6, true><<<g1, b1, 0, s>>>(d, g, p);
       }
     } else {
-      dim3 b1(128), g1((g.nx + 127) / 128, g.ny, g.nz);
-      switch (force_axis(p)) {
-        case 0: k_stream_collide<Q, 0><<<g1, b1, 0, s>>>(d, g, p); break;
-        case 1: k_stream_collide<Q, 1><<<g1, b1, 0, s>>>(d, g, p); break;
-        case 2: k_stream_collide<Q, 2><<<g1, b1, 0, s>>>(d, g, p); break;
-        default: k_stream_collide<Q, 3><<<g1, b1, 0, s>>>(d, g, p);
-      }
+      // (the turbulence model's form spills under a register bound)
+      if (p.les_cs > 0.0) bulk_fp64<4>(d, g, p, s);
+      else bulk_fp64<Q == 27 ? 16 : 20>(d, g, p, s);
     }
     return cudaGetLastError();
   }
