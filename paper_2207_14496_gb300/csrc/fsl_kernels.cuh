@@ -139,6 +139,46 @@ inline int force_axis(const Phys& p) {
   return n <= 1 ? a : 3;
 }
 
+// ---- FP64 additions near 1 on the integer pipes.  GB300 has two FP64 lanes per
+// SM and 128 integer lanes that the FP64 bulk pass leaves idle.  Its bracket
+// 1 + 3 cu + 4.5 cu^2 - 1.5 u.u adds terms below 1 to a value in [1/4, 2), which
+// fixed point carries exactly: a value is an integer times 2^-60 (its last FP64
+// place is bit 6, 7 or 8 of it), a term the floor of its multiple of 2^-60 and
+// whether anything lies below (sticky).  Rounding the integer sum at the place of
+// the result, ties to even, gives the correctly rounded sum, the same bits as
+// the FP64 addition.
+struct Fix60 {
+  unsigned long long x;  // floor(|v| 2^60)
+  unsigned sticky;       // 1 if |v| 2^60 is not that integer
+};
+// |v| < 1 (a zero or subnormal v reads as a sticky bit far below, which changes
+// no sum: the other operand has its last place above it)
+__device__ __forceinline__ Fix60 fix60(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int e = (int)(b >> 52) & 0x7ff;
+  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 7;
+  const int s = min(1022 - e, 63);
+  Fix60 f;
+  f.x = m >> s;
+  f.sticky = (f.x << s) != m ? 1u : 0u;
+  return f;
+}
+// bits below the last FP64 place of s 2^-60 in [1/4, 2)
+__device__ __forceinline__ int fix60_drop(unsigned long long s) {
+  return 6 + (int)min((unsigned)(s >> 32) >> 27, 2u);
+}
+// s (+ something below 1 if sticky) rounded to an FP64 number, ties to even
+__device__ __forceinline__ unsigned long long fix60_round(unsigned long long s, unsigned sticky) {
+  const int k = fix60_drop(s);
+  const unsigned half = 1u << (k - 1);
+  s += half - 1u + (sticky | (((unsigned)s >> k) & 1u));
+  return s & ~(unsigned long long)(2u * half - 1u);
+}
+__device__ __forceinline__ double fix60_double(unsigned long long s) {
+  const int k = fix60_drop(s);
+  return __longlong_as_double((long long)((s >> k) + ((unsigned long long)(1014 + k) << 52)));
+}
+
 // Collision (SRT or TRT) with Guo forcing (Eqs. nm-lbm-collision,
 // nm-lbm-force-guo) of the streamed FP64 values fin into fout.  Returns u.u
 // for the stability guard.
@@ -153,8 +193,12 @@ inline int force_axis(const Phys& p) {
 // a pair with no velocity component along it has one common force term and
 // no odd part.  Two FP64 lanes per SM make the operation count the time of
 // the FP64 bulk pass: D3Q27 TRT, force along z, 574 in place of 876 per cell,
-// and 160^3 of the drop impact takes 1.90 ms in place of 2.82.
-template <int Q, int AX>
+// and 160^3 of the drop impact takes 1.80 ms in place of 2.82.
+// FIXED (the bulk pass, which waits for the FP64 pipes; the interface pass waits
+// for its chain of operations): the six additions of a pair's two brackets run
+// on the integer pipes where |u| is small enough for their range: 160^3 drop
+// impact 1,981 -> 1,756 us per step, 400x400 wave 101 -> 91.
+template <int Q, int AX, bool FIXED = false>
 __device__ __forceinline__ double collide64(const double* fin, double* fout, const Phys& p,
                                             double& rho_out) {
   constexpr int NP = (Q - 1) / 2;
@@ -182,13 +226,38 @@ __device__ __forceinline__ double collide64(const double* fin, double* fout, con
   }
   double cu[NP], fe[Q];
   fe[0] = wr[0] * (1.0 - h);
+  // |cu| <= sqrt(3) |u| < 0.2122: 3 cu below 0.637, 4.5 cu^2 below 0.203 and
+  // 1.5 u.u below 0.023 keep every partial sum in [1/4, 2)
+  if (FIXED && usq < 0.015) {
+    const Fix60 fh = fix60(h);
+    const unsigned long long hn = 0ull - fh.x - fh.sticky;  // floor(-h 2^60)
+    constexpr unsigned long long one = 1ull << 60;
 #pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    const int i = 2 * k + 1;
-    cu[k] = dot3r<double>(dir_c(i, 0), dir_c(i, 1), dir_c(i, 2), u[0], u[1], u[2]);
-    const double c3 = 3.0 * cu[k], cc = 4.5 * cu[k] * cu[k];
-    fe[i] = wr[len2(i)] * ((1.0 + c3) + cc - h);
-    fe[i + 1] = wr[len2(i)] * ((1.0 - c3) + cc - h);
+    for (int k = 0; k < NP; ++k) {
+      const int i = 2 * k + 1;
+      cu[k] = dot3r<double>(dir_c(i, 0), dir_c(i, 1), dir_c(i, 2), u[0], u[1], u[2]);
+      const double c3 = 3.0 * cu[k], cc = 4.5 * cu[k] * cu[k];
+      const Fix60 f3 = fix60(c3), fc = fix60(cc);
+      const unsigned long long n3 = 0ull - f3.x - f3.sticky;
+      const bool neg = __double_as_longlong(c3) < 0;
+      const unsigned long long a =
+          fix60_round(fix60_round(fix60_round(one + (neg ? n3 : f3.x), f3.sticky) + fc.x, fc.sticky) + hn,
+                      fh.sticky);
+      const unsigned long long b =
+          fix60_round(fix60_round(fix60_round(one + (neg ? f3.x : n3), f3.sticky) + fc.x, fc.sticky) + hn,
+                      fh.sticky);
+      fe[i] = wr[len2(i)] * fix60_double(a);
+      fe[i + 1] = wr[len2(i)] * fix60_double(b);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const int i = 2 * k + 1;
+      cu[k] = dot3r<double>(dir_c(i, 0), dir_c(i, 1), dir_c(i, 2), u[0], u[1], u[2]);
+      const double c3 = 3.0 * cu[k], cc = 4.5 * cu[k] * cu[k];
+      fe[i] = wr[len2(i)] * ((1.0 + c3) + cc - h);
+      fe[i + 1] = wr[len2(i)] * ((1.0 - c3) + cc - h);
+    }
   }
   double om = p.omega, pre = p.pre_e, le = p.lam_e, lo = p.lam_o, pe = p.pre_e, po = p.pre_o;
   if (p.les_cs > 0.0) {
@@ -1374,7 +1443,7 @@ __global__ void __launch_bounds__(32, MINB) k_stream_collide(Dev d, Geom g, Phys
     nb.setup(g, x, y, z);
     R fin[Q], fout[Q], rho;
     pull_liquid<Q, ST>(A, P, d.flags, nb, c, (fl & F_NEAR_OBST) != 0, fin);
-    const R usq = collide64<Q, AX>(fin, fout, p, rho);
+    const R usq = collide64<Q, AX, true>(fin, fout, p, rho);
     if (!(usq < (R)(1.0 / 3.0))) bad = true;
 #pragma unroll
     for (int i = 0; i < Q; ++i) ST::stw(B + i * P + c, fout[i]);
