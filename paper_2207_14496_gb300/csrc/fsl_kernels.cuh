@@ -147,21 +147,55 @@ inline int force_axis(const Phys& p) {
 // whether anything lies below (sticky).  Rounding the integer sum at the place of
 // the result, ties to even, gives the correctly rounded sum, the same bits as
 // the FP64 addition.
+// Products with a full mantissa (3 cu, 4.5 cu^2, w rho times the bracket) are
+// rounded the same way from the integer product of the mantissas.
 struct Fix60 {
   unsigned long long x;  // floor(|v| 2^60)
   unsigned sticky;       // 1 if |v| 2^60 is not that integer
 };
-// |v| < 1 (a zero or subnormal v reads as a sticky bit far below, which changes
-// no sum: the other operand has its last place above it)
-__device__ __forceinline__ Fix60 fix60(double v) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-  const int e = (int)(b >> 52) & 0x7ff;
-  const unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 7;
-  const int s = min(1022 - e, 63);
+__device__ __forceinline__ unsigned long long mantissa(double v) {
+  return ((unsigned long long)__double_as_longlong(v) & 0xfffffffffffffull) | 0x10000000000000ull;
+}
+__device__ __forceinline__ int exponent(double v) {  // biased
+  return (int)((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ff;
+}
+// m 2^(e - 1075), m in [2^52, 2^53], below 1.  (A zero or subnormal number, whose
+// mantissa has no leading 1, reads as a sticky bit far below, which changes no
+// sum: the other operand has its last place above it.)
+__device__ __forceinline__ Fix60 fix60_of(unsigned long long m, int e) {
+  const int s = max(0, min(1022 - e, 63));
+  m <<= 7;
   Fix60 f;
   f.x = m >> s;
   f.sticky = (f.x << s) != m ? 1u : 0u;
   return f;
+}
+__device__ __forceinline__ Fix60 fix60(double v) { return fix60_of(mantissa(v), exponent(v)); }
+// floor(v 2^60) with the sign; top: largest |v| seen (upper word)
+__device__ __forceinline__ Fix60 fix60_signed(double v, unsigned& top) {
+  top = max(top, (unsigned)((unsigned long long)__double_as_longlong(v) >> 32) & 0x7fffffffu);
+  Fix60 f = fix60(v);
+  if (__double_as_longlong(v) < 0) f.x = 0ull - f.x - f.sticky;
+  return f;
+}
+// s / 2^d rounded, ties to even (sticky: something below the bits of s)
+__device__ __forceinline__ unsigned long long drop_bits(unsigned long long s, int d, unsigned sticky) {
+  const unsigned half = 1u << (d - 1);
+  return (s + (half - 1u + (sticky | (((unsigned)s >> d) & 1u)))) >> d;
+}
+// 3 cu and 4.5 cu cu (each product rounded), |cu| < 0.22
+__device__ __forceinline__ Fix60 fix60_3(double cu) {
+  const unsigned long long t = 3ull * mantissa(cu);  // 54 or 55 bits
+  const int d = 1 + (int)(t >> 54);
+  return fix60_of(drop_bits(t, d, 0u), exponent(cu) + d);
+}
+__device__ __forceinline__ Fix60 fix60_45(double cu) {
+  const unsigned long long m = mantissa(cu), t = 9ull * m;  // 56 or 57 bits
+  const int d = 3 + (int)(t >> 56), e = exponent(cu);
+  const unsigned long long a = drop_bits(t, d, 0u) << 10, b = m << 11;
+  const unsigned long long hi = __umul64hi(a, b);  // the product's upper 62 or 63 bits
+  const int k = 9 + (int)(hi >> 62);
+  return fix60_of(drop_bits(hi, k, a * b != 0ull ? 1u : 0u), k + d + 2 * e - 1033);
 }
 // bits below the last FP64 place of s 2^-60 in [1/4, 2)
 __device__ __forceinline__ int fix60_drop(unsigned long long s) {
@@ -177,6 +211,16 @@ __device__ __forceinline__ unsigned long long fix60_round(unsigned long long s, 
 __device__ __forceinline__ double fix60_double(unsigned long long s) {
   const int k = fix60_drop(s);
   return __longlong_as_double((long long)((s >> k) + ((unsigned long long)(1014 + k) << 52)));
+}
+// s 2^-60 times a positive normal number given by its mantissa << 11 and its
+// exponent, rounded
+__device__ __forceinline__ double fix60_mul(unsigned long long s, unsigned long long m, int e) {
+  const int k = fix60_drop(s);
+  const unsigned long long a = s << (11 - k);
+  const unsigned long long hi = __umul64hi(a, m);  // the product's upper 63 or 64 bits
+  const int d = 10 + (int)(hi >> 63);
+  return __longlong_as_double((long long)(drop_bits(hi, d, a * m != 0ull ? 1u : 0u) +
+                                          ((unsigned long long)(d + k + e - 19) << 52)));
 }
 
 // Collision (SRT or TRT) with Guo forcing (Eqs. nm-lbm-collision,
@@ -195,15 +239,34 @@ __device__ __forceinline__ double fix60_double(unsigned long long s) {
 // the FP64 bulk pass: D3Q27 TRT, force along z, 574 in place of 876 per cell,
 // and 160^3 of the drop impact takes 1.80 ms in place of 2.82.
 // FIXED (the bulk pass, which waits for the FP64 pipes; the interface pass waits
-// for its chain of operations): the six additions of a pair's two brackets run
-// on the integer pipes where |u| is small enough for their range: 160^3 drop
-// impact 1,981 -> 1,756 us per step, 400x400 wave 101 -> 91.
+// for its chain of operations): the density sum and the equilibria of a pair
+// (six additions, five products) run on the integer pipes where |u| is small
+// enough for their range.  160^3 drop impact, us per step: 1,981 without, 1,756
+// with the additions of the brackets, 1,512 with all of it (and 12 warps per SM
+// in place of 16); 400x400 wave: 101, 91, 86.
 template <int Q, int AX, bool FIXED = false>
 __device__ __forceinline__ double collide64(const double* fin, double* fout, const Phys& p,
                                             double& rho_out) {
   constexpr int NP = (Q - 1) / 2;
   double rho, drho, j[3];
-  density<Q, false, double>(fin, rho, drho);
+  bool summed = false;
+  if (FIXED) {
+    // the density, left to right: near equilibrium f_0 (8/27 or 1/3 of rho) puts
+    // the partial sums in [1/4, 2); if they leave it, FP64 additions below
+    unsigned top = 0u;
+    const Fix60 f0 = fix60_signed(fin[0], top);
+    unsigned long long sum = f0.x;
+    bool in = (sum >> 58) - 1u < 7u && f0.sticky == 0u;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      const Fix60 f = fix60_signed(fin[i], top);
+      sum = fix60_round(sum + f.x, f.sticky);
+      in = in && (sum >> 58) - 1u < 7u;
+    }
+    summed = in && top < 0x3ff00000u;  // every |f_i| below 1
+    rho = fix60_double(sum);
+  }
+  if (!summed) density<Q, false, double>(fin, rho, drho);
   momentum<Q, double>(fin, j[0], j[1], j[2]);
   // Eq. nm-lbm-velocity with F = rho g: u = j / rho + g / 2
   double u[3], F[3];
@@ -228,7 +291,8 @@ __device__ __forceinline__ double collide64(const double* fin, double* fout, con
   fe[0] = wr[0] * (1.0 - h);
   // |cu| <= sqrt(3) |u| < 0.2122: 3 cu below 0.637, 4.5 cu^2 below 0.203 and
   // 1.5 u.u below 0.023 keep every partial sum in [1/4, 2)
-  if (FIXED && usq < 0.015) {
+  // (rho within a factor of 4 of 1: wr is normal)
+  if (FIXED && usq < 0.015 && rho > 0.25 && rho < 4.0) {
     const Fix60 fh = fix60(h);
     const unsigned long long hn = 0ull - fh.x - fh.sticky;  // floor(-h 2^60)
     constexpr unsigned long long one = 1ull << 60;
@@ -236,18 +300,19 @@ __device__ __forceinline__ double collide64(const double* fin, double* fout, con
     for (int k = 0; k < NP; ++k) {
       const int i = 2 * k + 1;
       cu[k] = dot3r<double>(dir_c(i, 0), dir_c(i, 1), dir_c(i, 2), u[0], u[1], u[2]);
-      const double c3 = 3.0 * cu[k], cc = 4.5 * cu[k] * cu[k];
-      const Fix60 f3 = fix60(c3), fc = fix60(cc);
+      const Fix60 f3 = fix60_3(cu[k]), fc = fix60_45(cu[k]);
       const unsigned long long n3 = 0ull - f3.x - f3.sticky;
-      const bool neg = __double_as_longlong(c3) < 0;
+      const bool neg = __double_as_longlong(cu[k]) < 0;
+      const unsigned long long wm = mantissa(wr[len2(i)]) << 11;
+      const int we = exponent(wr[len2(i)]);
       const unsigned long long a =
           fix60_round(fix60_round(fix60_round(one + (neg ? n3 : f3.x), f3.sticky) + fc.x, fc.sticky) + hn,
                       fh.sticky);
       const unsigned long long b =
           fix60_round(fix60_round(fix60_round(one + (neg ? f3.x : n3), f3.sticky) + fc.x, fc.sticky) + hn,
                       fh.sticky);
-      fe[i] = wr[len2(i)] * fix60_double(a);
-      fe[i + 1] = wr[len2(i)] * fix60_double(b);
+      fe[i] = fix60_mul(a, wm, we);
+      fe[i + 1] = fix60_mul(b, wm, we);
     }
   } else {
 #pragma unroll
@@ -3451,7 +3516,7 @@ struct Kernels {
     } else {
       // (the turbulence model's form spills under a register bound)
       if (p.les_cs > 0.0) bulk_fp64<4>(d, g, p, s);
-      else bulk_fp64<Q == 27 ? 16 : 20>(d, g, p, s);
+      else bulk_fp64<Q == 27 ? 12 : 20>(d, g, p, s);
     }
     return cudaGetLastError();
   }
