@@ -332,6 +332,10 @@ fsl_status copy_field(fsl_handle* h, const void* dev, size_t elem, void* host) {
 }
 
 const size_t kGraphChunk = 64;
+// Steps of a small domain per launch (k_steps): a few steps do not repay the
+// instruction fetch that a launch saves, and a launch should not hold the GPU
+// for more than some ten milliseconds.
+const int kStepsMin = 4, kStepsMost = 512;
 // The interface list is put back into memory order (k_sort_interface) every so
 // many steps: inside the captured graphs of that many steps or more, before
 // the next launch where shorter ones have added up.  Every step of churn costs: bubbly
@@ -488,6 +492,13 @@ fsl_status fsl_step(fsl_handle* h, int nsteps) {
   }
   int left = nsteps;
   while (left > 0) {
+    if (left >= kStepsMin && h->L->small_domain(h->g)) {
+      const int n = std::min(left, kStepsMost);
+      FSL_CK(h->L->steps(h->d, h->g, h->p, n, h->stream));
+      h->since_sort += n;
+      left -= n;
+      continue;
+    }
     const int chunk = left >= (int)kGraphChunk ? (int)kGraphChunk : left;
     auto it = h->graphs.find(chunk);
     if (it == h->graphs.end()) {

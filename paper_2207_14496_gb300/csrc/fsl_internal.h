@@ -184,6 +184,9 @@ struct Launch {
   int (*launches_per_step)(const Geom&);
   // one time step of n members (one launch per kernel for all of them)
   cudaError_t (*batch_step)(const MemberTable& t, int n, const BatchGrid& bg, cudaStream_t);
+  // whether a domain's steps run in one launch, and that launch (n steps)
+  bool (*small_domain)(const Geom&);
+  cudaError_t (*steps)(const Dev&, const Geom&, const Phys&, int n, cudaStream_t);
 };
 
 // Launch tables, one translation unit per (storage, lattice).

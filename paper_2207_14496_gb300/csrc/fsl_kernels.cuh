@@ -1479,6 +1479,28 @@ __global__ void __launch_bounds__(128, 3) k_stream_collide_pp(Dev d, Geom g, Phy
 namespace fsl {
 
 // ------------------------------------------------------------ stream-collide
+// Streaming and collision of cell (x, y, z) in FP64 if it is liquid; returns
+// whether it reached |u|^2 >= 1/3.
+template <int Q, class ST, int AX>
+__device__ __forceinline__ bool bulk64_cell(const Dev& d, const Geom& g, const Phys& p, int x, int y,
+                                            int z) {
+  const int cur = d.ctrl->step & 1;  // pdf[step & 1] holds f*(t)
+  const double* A = (const double*)d.pdf[cur];
+  double* B = (double*)d.pdf[cur ^ 1];
+  const long long P = g.plane;
+  const int c = x + g.sx * (y + g.ny * z);
+  const uint8_t fl = (x < g.nx) ? d.flags[c] : (uint8_t)T_GAS;
+  if ((fl & F_TYPE) != T_LIQ) return false;
+  Nbr nb;
+  nb.setup(g, x, y, z);
+  double fin[Q], fout[Q], rho;
+  pull_liquid<Q, ST>(A, P, d.flags, nb, c, (fl & F_NEAR_OBST) != 0, fin);
+  const double usq = collide64<Q, AX, true>(fin, fout, p, rho);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) ST::stw(B + i * P + c, fout[i]);
+  return !(usq < 1.0 / 3.0);
+}
+
 // FP64 pass over all cells: liquid cells stream and collide here (interface cells
 // are handled by k_stream_collide_if from the step's interface list).
 // One warp per block, 32 cells of a row: blocks of 128 cells left warps of a
@@ -1489,31 +1511,10 @@ namespace fsl {
 // 1,981 so.)
 template <int Q, int AX, int MINB>
 __global__ void __launch_bounds__(32, MINB) k_stream_collide(Dev d, Geom g, Phys p) {
-  using ST = SF64;
-  using T = double;
-  using R = double;
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
-  const int cur = ctrl->step & 1;  // pdf[step & 1] holds f*(t)
-  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
-  const T* __restrict__ A = (const T*)d.pdf[cur];
-  T* __restrict__ B = (T*)d.pdf[cur ^ 1];
-  const long long P = g.plane;
-  const int c = x + g.sx * (y + g.ny * z);
-  const uint8_t fl = (x < g.nx) ? d.flags[c] : (uint8_t)T_GAS;
-  const int type = fl & F_TYPE;
-  bool bad = false;
-  if (type == T_LIQ) {
-    Nbr nb;
-    nb.setup(g, x, y, z);
-    R fin[Q], fout[Q], rho;
-    pull_liquid<Q, ST>(A, P, d.flags, nb, c, (fl & F_NEAR_OBST) != 0, fin);
-    const R usq = collide64<Q, AX, true>(fin, fout, p, rho);
-    if (!(usq < (R)(1.0 / 3.0))) bad = true;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) ST::stw(B + i * P + c, fout[i]);
-  }
-  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0)
+  const bool bad = bulk64_cell<Q, SF64, AX>(d, g, p, blockIdx.x * 32 + threadIdx.x, blockIdx.y, blockIdx.z);
+  if (__any_sync(0xffffffffu, bad) && threadIdx.x == 0)
     atomicCAS(&ctrl->unstable_step, -1, ctrl->step + 1);
 }
 
@@ -1735,7 +1736,7 @@ __device__ __forceinline__ void stream_collide_col_body(const Dev& d, const Geom
     if (nb.Y[2] < 0) { cross |= dirs_with<Q>(1, -1); nb.Y[2] = y; }
     if (nb.Z[0] < 0) { cross |= dirs_with<Q>(2, 1); nb.Z[0] = z; }
     if (nb.Z[2] < 0) { cross |= dirs_with<Q>(2, -1); nb.Z[2] = z; }
-    const R* __restrict__ phi = phi_work<R>(d);
+    const R* phi = phi_work<R>(d);
     R own[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) own[i] = ST::ldw(A + i * P + c);
@@ -1744,7 +1745,7 @@ __device__ __forceinline__ void stream_collide_col_body(const Dev& d, const Geom
       const int n = nb.in(-dir_c(i, 0), -dir_c(i, 1), -dir_c(i, 2));
       const uint8_t b = d.flags[n];
       col.fin[i - 1][tid] = ST::ldw(A + i * P + n);
-      col.phi[i - 1][tid] = phi[n];
+      col.phi[i - 1][tid] = ld_const<ST>(phi + n);
       col.fb[i - 1][tid] = (cross >> i) & 1u ? (uint8_t)T_OBST : b;
     }
     if (cross && g.free_slip) {
@@ -2864,9 +2865,10 @@ __device__ inline int block_max(int v, int* sh) {
   return r;
 }
 
-// Sum of v and maxima of a and b over a block of 256 threads, in the tree of
-// block_sum and block_max (thread t takes t + 128, t + 64, ..., t + 1), the
-// three together and the last five levels by shuffles; in thread 0.
+// Sum of v and maxima of a and b over the NT threads of a block, in the tree of
+// block_sum and block_max (thread t takes t + NT / 2, ..., t + 1), the three
+// together and the last five levels by shuffles; in thread 0.
+template <int NT>
 __device__ __forceinline__ void block_reduce3(double& v, int& a, int& b, double* shd, int* sha,
                                               int* shb) {
   const int t = threadIdx.x;
@@ -2875,7 +2877,7 @@ __device__ __forceinline__ void block_reduce3(double& v, int& a, int& b, double*
   shb[t] = b;
   __syncthreads();
 #pragma unroll
-  for (int s = 128; s >= 32; s >>= 1) {
+  for (int s = NT / 2; s >= 32; s >>= 1) {
     if (t < s) {
       shd[t] = v = v + shd[t + s];
       sha[t] = a = max(a, sha[t + s]);
@@ -2898,16 +2900,20 @@ __device__ __forceinline__ void block_reduce3(double& v, int& a, int& b, double*
 // fixed tree order), whatever the number of blocks that work on them; the
 // last block to finish combines the partials in part order and advances the
 // counters.  A handle that never traces needs none of that: block 0 alone
-// advances the counters.
+// advances the counters (not in k_steps, whose blocks may still wait at the
+// barrier before).  The tree of a part is that of 256 threads; a block of 128
+// adds its first level in the thread.
 constexpr int kEndBlocks = 64;
+template <int NT, bool ALONE>
 __device__ __forceinline__ void end_step_body(const Dev& d, const Geom& g) {
-  __shared__ double shd[256];
-  __shared__ int sha[256], shb[256];
+  static_assert(NT == 256 || NT == 128, "");
+  __shared__ double shd[NT];
+  __shared__ int sha[NT], shb[NT];
   __shared__ bool last;
   Ctrl* ctrl = d.ctrl;
   if (frozen(ctrl)) return;
   const int every = ctrl->trace_every;
-  if (every == 0 && blockIdx.x != 0) return;
+  if (ALONE && every == 0 && blockIdx.x != 0) return;
   const bool tracing = every > 0 && ((ctrl->step + 1) % every) == 0;
   double* part = d.red;                         // kEndBlocks column partials
   int* ipart = reinterpret_cast<int*>(d.red + kEndBlocks);  // 2 x kEndBlocks maxima
@@ -2920,19 +2926,24 @@ __device__ __forceinline__ void end_step_body(const Dev& d, const Geom& g) {
       const int k0 = vb * chunk, k1 = min(ncol, k0 + chunk);
       double s = 0.0;
       int hbest = -1;
-      for (int k = k0 + threadIdx.x; k < k1; k += 256) {
-        const long long cidx = (long long)g.sx * k;   // cell (0, j, kz), k = j + ny kz
-        s += d.phi[cidx];
-        if ((d.flags[cidx] & F_TYPE) == T_IF) hbest = max(hbest, k % g.ny);
+#pragma unroll
+      for (int h = 0; h < 256; h += NT) {
+        double sh = 0.0;
+        for (int k = k0 + threadIdx.x + h; k < k1; k += 256) {
+          const long long cidx = (long long)g.sx * k;   // cell (0, j, kz), k = j + ny kz
+          sh += d.phi[cidx];
+          if ((d.flags[cidx] & F_TYPE) == T_IF) hbest = max(hbest, k % g.ny);
+        }
+        s = h == 0 ? sh : s + sh;
       }
       // front: cells (i, 0, kz)
       const int r0 = vb * rchunk, r1 = min(nrow, r0 + rchunk);
       int fbest = -1;
-      for (int k = r0 + threadIdx.x; k < r1; k += 256) {
+      for (int k = r0 + threadIdx.x; k < r1; k += NT) {
         const int i = k % g.nx, kz = k / g.nx;
         if ((d.flags[i + (long long)g.sx * g.ny * kz] & F_TYPE) == T_IF) fbest = max(fbest, i);
       }
-      block_reduce3(s, fbest, hbest, shd, sha, shb);
+      block_reduce3<NT>(s, fbest, hbest, shd, sha, shb);
       if (threadIdx.x == 0) {
         part[vb] = s;
         ipart[vb] = fbest;
@@ -2940,7 +2951,7 @@ __device__ __forceinline__ void end_step_body(const Dev& d, const Geom& g) {
       }
     }
   }
-  if (every > 0) {
+  if (!ALONE || every > 0) {
     __threadfence();
     if (threadIdx.x == 0) last = atomicAdd(&ctrl->end_blocks, 1u) == gridDim.x - 1;
     __syncthreads();
@@ -2952,7 +2963,7 @@ __device__ __forceinline__ void end_step_body(const Dev& d, const Geom& g) {
     double cp = in ? *(volatile double*)&part[threadIdx.x] : 0.0;
     int fp = in ? *(volatile int*)&ipart[threadIdx.x] : -1;
     int hp = in ? *(volatile int*)&ipart[kEndBlocks + threadIdx.x] : -1;
-    block_reduce3(cp, fp, hp, shd, sha, shb);
+    block_reduce3<NT>(cp, fp, hp, shd, sha, shb);
     if (threadIdx.x == 0) {
       shd[0] = cp;
       sha[0] = fp;
@@ -2980,17 +2991,69 @@ __device__ __forceinline__ void end_step_body(const Dev& d, const Geom& g) {
     ctrl->n_emptied = 0;
     ctrl->end_blocks = 0;
     ctrl->n_tiles = 0;
-    ctrl->bar = 0;
+    if (ALONE) ctrl->bar = 0;
     __threadfence();
     ctrl->step += 1;
   }
 }
-static __global__ void __launch_bounds__(256) k_end_step(Dev d, Geom g) { end_step_body(d, g); }
+static __global__ void __launch_bounds__(256) k_end_step(Dev d, Geom g) { end_step_body<256, true>(d, g); }
 static __global__ void __launch_bounds__(256) kb_end_step(MemberTable t) {
   FSL_MEMBER(t);
-  end_step_body(d, g);
+  end_step_body<256, true>(d, g);
 }
 
+
+// ------------------------------------------------------------ whole steps
+// n steps of a small domain in one cooperative launch: the phases of the
+// separate kernels, separated by grid-wide barriers.  In a small domain each of
+// those kernels is one or two warps per SM that run once through thousands of
+// instructions, and every launch fetches them anew (about 340 cycles per 128
+// bytes); here they stay in the SMs' instruction caches from step to step, and
+// six barriers take the place of five launches (small_domain has the figures).
+constexpr int kStepsThreads = 128;
+template <int Q, class STO, int AX>
+__global__ void __launch_bounds__(kStepsThreads) k_steps(Dev d, Geom g, Phys p, int n) {
+  using ST = Coherent<STO>;
+  Ctrl* ctrl = d.ctrl;
+  const unsigned nb = gridDim.x;
+  unsigned bar = 0;  // arrivals the next barrier waits for (the host clears ctrl->bar afterwards)
+  for (int s = 0; s < n; ++s) {
+    if (frozen(ctrl)) return;  // the same for every block: latched steps end before the barrier
+    // interface pass, and the bulk pass from the last warp of the grid on
+    if constexpr (Q == 19) stream_collide_col_body<Q, ST, AX>(d, g, p);
+    else stream_collide_if_body<Q, ST, AX>(d, g, p);
+    {
+      constexpr int W = STO::kShift ? 64 : 32;  // cells of a warp
+      const int lane = threadIdx.x & 31;
+      const unsigned warps = nb * (kStepsThreads / 32);
+      const unsigned ntx = (unsigned)((g.nx + W - 1) / W), units = ntx * g.ny * g.nz;
+      bool bad = false;
+      for (unsigned u = warps - 1u - ((threadIdx.x >> 5) * nb + blockIdx.x); u < units; u += warps) {
+        const int x0 = (int)(u % ntx) * W, row = (int)(u / ntx);
+        if constexpr (STO::kShift)
+          bad |= pair_update<Q, ST, true, true>(d, g, p, x0 + 2 * lane, row % g.ny, row / g.ny, lane);
+        else
+          bad |= bulk64_cell<Q, ST, AX>(d, g, p, x0 + lane, row % g.ny, row / g.ny);
+      }
+      if (__any_sync(0xffffffffu, bad) && lane == 0)
+        atomicCAS(&ctrl->unstable_step, -1, ctrl->step + 1);
+    }
+    if (!grid_barrier(ctrl, bar += nb)) return;
+    fill_body<Q>(d, g);
+    empty_body<Q, ST>(d, g);
+    commit_phi_body(d);
+    if (!grid_barrier(ctrl, bar += nb)) return;
+    finalise_share_body<Q>(d, g);
+    refill_body<Q, ST>(d, g, p);
+    if (!grid_barrier(ctrl, bar += nb)) return;
+    excess_gather_body<Q>(d, g);
+    if (!grid_barrier(ctrl, bar += nb)) return;
+    classify_body<Q, ST>(d, g, p);
+    if (!grid_barrier(ctrl, bar += nb)) return;
+    end_step_body<kStepsThreads, false>(d, g);
+    if (s + 1 < n && !grid_barrier(ctrl, bar += nb)) return;
+  }
+}
 
 // ------------------------------------------------------------ initialisation
 static __global__ void k_ctrl_reset(Ctrl* ctrl, int trace_every) {
@@ -3219,6 +3282,61 @@ struct Kernels {
     k_classify<Q, ST><<<kCellListBlocks, 128, 0, s>>>(d, g, p);
     k_end_step<<<kEndBlocks, 256, 0, s>>>(d, g);
     return cudaGetLastError();
+  }
+  // Domains that step in one launch of k_steps: no bubble model, the default
+  // bulk variant, and few enough (padded) cells for one block of 128 threads per
+  // SM, by measured step times (us, separate launches / k_steps): D3Q19 FP32
+  // 64x64x1 39 / 28, 200x200x4 34 / 27, 400x400x1 41 / 33, dam break 120x80x8
+  // 45 / 38, FP16 the same; D3Q27 FP16 32^3 51 / 49 but 48^3 54 / 62; D3Q19 FP64
+  // 33x33 47 / 39, 64x64 62 / 58, 150x150 52 / 45 but 128x128x2 64 / 67 and
+  // 750x200 with the turbulence model 75 / 101; D3Q27 FP64 32^3 82 / 109 (the
+  // FP64 chains of few warps bound those).
+  static constexpr long long kSmallCells =
+      ST::kShift ? (Q == 19 ? 200000 : 40000) : (Q == 19 ? 25000 : 0);
+  static bool small_domain(const Geom& g) {
+    return g.cells <= kSmallCells && !g.bubbles && g.variant == 0;
+  }
+  static cudaError_t steps(const Dev& d, const Geom& g, const Phys& p, int n, cudaStream_t s) {
+    if constexpr (kSmallCells == 0) {
+      return cudaErrorNotSupported;
+    } else {
+      // FP64: the axis that gravity has in the plane workloads, or the general form
+      if constexpr (!ST::kShift)
+        if (force_axis(p) == 1) return steps_as<1>(d, g, p, n, s);
+      return steps_as<3>(d, g, p, n, s);
+    }
+  }
+  template <int AX>
+  static cudaError_t steps_as(const Dev& d, const Geom& g, const Phys& p, int n, cudaStream_t s) {
+    static int sms = 0;
+    if (sms == 0) {
+      cudaError_t e = cudaFuncSetAttribute(k_steps<Q, ST, AX>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIfSmem);
+      if (e != cudaSuccess) return e;
+      int per_sm = 0, dev = 0, k = 0;
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_steps<Q, ST, AX>, kStepsThreads, kIfSmem);
+      if (e == cudaSuccess) e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&k, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return e;
+      if (per_sm < 1) return cudaErrorLaunchOutOfResources;
+      sms = k;
+    }
+    // a block per kStepsThreads cells, at most one per SM
+    const long long want = (g.cells + kStepsThreads - 1) / kStepsThreads;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.gridDim = dim3((unsigned)(want < sms ? want : sms));
+    cfg.blockDim = dim3(kStepsThreads);
+    cfg.dynamicSmemBytes = kIfSmem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_steps<Q, ST, AX>, d, g, p, n);
+    // its barrier arrivals
+    if (e == cudaSuccess) e = cudaMemsetAsync(&d.ctrl->bar, 0, sizeof(unsigned), s);
+    return e;
   }
   static constexpr size_t kIfSmem = Q == 19 ? sizeof(IfColumn<Q, typename ST::R>) : 0;
   template <int AX>
@@ -3553,7 +3671,8 @@ struct Kernels {
   }
   static const Launch* table() {
     static const Launch L = {&step, &init, &total_mass, &max_velocity, &export_pdf,
-                             &pre_bulk, &stream_collide, &launches, &batch_step};
+                             &pre_bulk, &stream_collide, &launches, &batch_step,
+                             &small_domain, &steps};
     return &L;
   }
 };

@@ -216,6 +216,43 @@ struct SBF16 {
   }
 };
 
+// The same storage with loads that see what other SMs wrote earlier in the same
+// kernel (from L2), for the kernel that runs whole steps (k_steps); the loads
+// above may come from the non-coherent cache.
+template <class S>
+struct IsCoherent : std::false_type {};
+template <class S>
+struct Coherent : S {
+  using T = typename S::T;
+  using R = typename S::R;
+  static __device__ __forceinline__ R ldw(const T* p) {
+    if constexpr (std::is_same_v<T, __half>) return __half2float(__ldcg(p)) * S::kInv;
+    else if constexpr (std::is_same_v<T, __nv_bfloat16>) return __bfloat162float(__ldcg(p));
+    else return __ldcg(p);
+  }
+  static __device__ __forceinline__ float ld1(const T* p) {
+    if constexpr (std::is_same_v<T, __half>) return __half2float(__ldcg(p));
+    else if constexpr (std::is_same_v<T, __nv_bfloat16>) return __bfloat162float(__ldcg(p));
+    else return (float)__ldcg(p);
+  }
+  static __device__ __forceinline__ float2 ld2(const T* p) {
+    if constexpr (std::is_same_v<T, __half>)
+      return __half22float2(__ldcg(reinterpret_cast<const __half2*>(p)));
+    else if constexpr (std::is_same_v<T, __nv_bfloat16>)
+      return __bfloat1622float2(__ldcg(reinterpret_cast<const __nv_bfloat162*>(p)));
+    else
+      return __ldcg(reinterpret_cast<const float2*>(p));
+  }
+};
+template <class S>
+struct IsCoherent<Coherent<S>> : std::true_type {};
+// A value that no kernel but k_steps writes while others read it.
+template <class ST, class R>
+__device__ __forceinline__ R ld_const(const R* p) {
+  if constexpr (IsCoherent<ST>::value) return *p;
+  else return __ldg(p);
+}
+
 // ----------------------------------------------------------------- geometry
 __device__ __forceinline__ void cell_xyz(const Geom& g, int c, int& x, int& y, int& z) {
   x = c % g.sx;
