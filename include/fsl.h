@@ -120,7 +120,8 @@ fsl_status fsl_workspace_bytes(const fsl_config* cfg, size_t* bytes);
  * out: receives the host handle (release with fsl_destroy).  The handle
  * creates one high-priority side stream and two events of its own (no device
  * memory): each step runs its interface-cell pass there, forked from and
- * joined back to the bound stream, beside the bulk pass; fsl_destroy
+ * joined back to the bound stream, beside the bulk pass, and with the bubble
+ * model the classes and curvature beside the bubble update; fsl_destroy
  * releases them. */
 fsl_status fsl_create(const fsl_config* cfg, void* d_workspace, size_t bytes, void* cuda_stream,
                       fsl_handle** out);

@@ -35,8 +35,7 @@
 // other cells keep whatever they held.  The parameter gradients are summed in
 // FP64, per block first and then with one atomic per block: one atomic per
 // thread put 130,000 additions to the same four addresses in the way of each
-// step (collision kernel of a 128x64x4 wave: 397 us, now 37 us with the
-// rest of the changes described at k_adj_collide).
+// step (k_adj_collide has the figures).
 #pragma once
 // Included by fsl_api.cu after fsl_kernels.cuh.
 
@@ -351,8 +350,9 @@ __device__ __forceinline__ void adj_collide_sums(const double* lfn, const double
 // What bounded it: the q-long arrays of a cell lived in local memory (loops
 // over directions that were not unrolled), 57 divisions per cell, and one
 // FP64 atomic per thread and parameter.  128x64x4 D3Q19 FP64 wave: 397 us and
-// 7 us for the separate mass kernel before; the FP64 sums (16,000 fluid cells
-// of about 700 FP64 operations on two lanes per SM) are what is left.
+// 7 us for the separate mass kernel before, 70 us now; the FP64 sums (16,000
+// fluid cells of about 700 FP64 operations on two lanes per SM) are what is
+// left.
 template <int Q, class ST>
 __global__ void __launch_bounds__(kAdjThreads)
     k_adj_collide(Geom g, Phys p, AdjLevel L0, AdjLevel L1, AdjFields<typename ST::R> A) {

@@ -153,7 +153,8 @@ struct BatchGrid {
 // Per-precision-family launch table, implemented in fsl_prec_*.cu.
 // Side stream and events of a handle: the interface pass of a step runs on
 // `side`, forked from and joined back to the step's stream, concurrently with
-// the bulk pass (the two write disjoint cells).  side == nullptr: one stream.
+// the bulk pass (the two write disjoint cells), and with the bubble model so
+// does classify beside the bubble update.  side == nullptr: one stream.
 struct Aux {
   cudaStream_t side;
   cudaEvent_t fork, join;
