@@ -314,7 +314,8 @@ __device__ __forceinline__ bool bulk_pair(const typename ST::T* __restrict__ A,
 
 // MULTI: tiles of rt.rows whole rows of a plane (rows of at most 128 cells);
 // else tiles of 256 cells of one row.  A 64-cell row fills only a quarter of
-// a one-row tile's lanes: 64x64x640, D3Q19, FP32, tube of obstacles, 278 us with one-row tiles' pair kernel, 106 us here.
+// a one-row tile's lanes: 64x64x640, D3Q19, FP32, tube of obstacles, 278 us with
+// the pair kernel on one-row tiles, 106 us here.
 template <int Q, class ST, int NS, int MINB, bool MULTI>
 __global__ void __launch_bounds__(kBulkThreads, MINB)
     k_stream_collide_bulk(Dev d, Geom g, Phys p, int ntx, RowTiles rt) {
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
   T* __restrict__ B = (T*)d.pdf[cur ^ 1];
   const long long P = g.plane;
   const int ntl = (int)ctrl->n_tiles;
-  if ((int)blockIdx.x >= ntl) return;
+  if (!MULTI && (int)blockIdx.x >= ntl) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < D; ++s) {
@@ -348,12 +349,26 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
 
   if (warp == kBulkConsumers) {
     // ---------------- producer warp: lane 0 waits for the stage and arms its
-    // barrier, lane i < Q copies direction i, lane Q the flags
+    // barrier, lane i < Q copies direction i, lane Q the flags.
+    // MULTI: the tiles of the first filling of the ring are the block's own,
+    // the others are claimed from a counter, because tiles of several rows
+    // differ in the liquid that they hold (steps: 64x64x640 FP32 Taylor bubble
+    // 256 -> 245 us, 48x48x480 177 -> 171).  The claim of the tile after the next and
+    // the list entry of the next are in flight while the producer waits for a
+    // stage.  Tiles of one row keep equal shares: claimed, their reads moved
+    // apart (256^3 drop impact -1.5 %, but 160^3 and 200^3 FP32 +3 %).
     int issued = 0;
     bool stop = false;
+    int k = MULTI && (int)blockIdx.x < ntl ? d.l_tiles[blockIdx.x] : -1;
+    int ahead = 0;
+    auto next_tile = [&](int j) {  // list entry of the block's tile j + 1, -1: none
+      const int claimed = __shfl_sync(0xffffffffu, ahead, 0);
+      const int ti = j + 1 < D ? (int)(blockIdx.x + (j + 1) * gridDim.x) : claimed;
+      if (lane == 0 && j + 2 >= D) ahead = (int)(D * gridDim.x + atomicAdd(&ctrl->tile_next, 1u));
+      return ti < ntl ? d.l_tiles[ti] : -1;
+    };
     for (int j = 0;; ++j) {
-      const int ti = blockIdx.x + j * gridDim.x;
-      if (ti >= ntl) break;
+      if (!MULTI && (int)(blockIdx.x + j * gridDim.x) >= ntl) break;
       const int s = j % D;
       int go = 1;
       if (lane == 0) {
@@ -367,9 +382,16 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
         stop = true;
         break;
       }
-      const int k = d.l_tiles[ti];
+      if (!MULTI) k = d.l_tiles[blockIdx.x + j * gridDim.x];
       unsigned char* stage = smem + (size_t)s * RING::stage_bytes;
       if constexpr (MULTI) {
+        if (k < 0) {  // no tile left: tell the consumers
+          if (lane == 0) {
+            tile_of[s] = make_int4(-1, 0, 0, 0);
+            mbar_arrive(&full[s]);
+          }
+          break;
+        }
         const int z = k / rt.per, y0 = (k % rt.per) * rt.rows;
         const int R = g.ny - y0 < rt.rows ? g.ny - y0 : rt.rows;
         const unsigned row_bytes = (unsigned)(g.sx * sizeof(T));
@@ -400,6 +422,7 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
                         (unsigned)(R * g.sx), &full[s]);
         }
         ++issued;
+        k = next_tile(j);
         continue;
       }
       const int x0 = (k % ntx) * kBulkTX;
@@ -435,6 +458,13 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
       const int first = issued > D ? issued - D : 0;
       for (int j = first; j < issued; ++j) mbar_wait(&full[j % D], (j / D) & 1);
     }
+    if (MULTI && lane == 0) {  // the last block to end its claims clears the counters
+      __threadfence();
+      if (atomicAdd(&ctrl->tile_done, 1u) == gridDim.x - 1) {
+        ctrl->tile_next = 0;
+        ctrl->tile_done = 0;
+      }
+    }
     return;
   }
 
@@ -444,8 +474,7 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
   const int rt_r = MULTI ? 2 * t / g.sx : 0;  // row of the tile the thread's cells lie in
   bool bad = false;
   for (int j = 0;; ++j) {
-    const int ti = blockIdx.x + j * gridDim.x;
-    if (ti >= ntl) break;
+    if (!MULTI && (int)(blockIdx.x + j * gridDim.x) >= ntl) break;
     const int s = j % D;
     const bool ok = mbar_wait(&full[s], (j / D) & 1);
     // the decision to stop is taken by the whole warp
@@ -460,6 +489,7 @@ __global__ void __launch_bounds__(kBulkThreads, MINB)
     const int4 tc = tile_of[s];
     const uchar2 f2 = *reinterpret_cast<const uchar2*>(stage + RING::pdf_bytes + 2 * t);
     if constexpr (MULTI) {
+      if (tc.x < 0) break;  // no tile left
       // (the cells of a row's padding hold the gas type)
       if (rt_r < tc.x)
         bad |= bulk_pair<Q, ST>(A, B, reinterpret_cast<const T*>(stage), kBulkSeg,

@@ -41,8 +41,8 @@ struct Ctrl {
   unsigned end_blocks; // end-of-step blocks finished
   unsigned n_tiles;    // tiles holding liquid cells, listed this step (16/32-bit path)
   unsigned n_if_next;  // interface cells of the next step (appended by k_classify)
-  unsigned tile_next;  // next tile handed out by the dynamically scheduled bulk kernel
-  unsigned tile_done;  // blocks of that kernel finished (the last one resets both)
+  unsigned tile_next;  // next tile handed out by the dynamically scheduled bulk kernels
+  unsigned tile_done;  // blocks of such a kernel finished (the last one resets both)
   unsigned bar;        // block arrivals at the grid barriers of the conversion kernel
                        // (reset by the end-of-step kernel)
 };
