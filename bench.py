@@ -470,9 +470,10 @@ def main():
 
 # FP64 instructions per liquid-cell update of the FP64 stream-collide kernel
 # for D3Q27 TRT with Guo forcing: ncu's smsp__sass_thread_inst_executed_op_
-# fp64_pred_on.sum (1.3365e9) over the liquid cells (1.526e6) of one launch
-# on the 160^3 drop impact.
-FP64_INSTR_PER_LIQUID_CELL_D3Q27_TRT = 876
+# fp64_pred_on.sum (6.629e8) over the liquid cells (1.526e6) of one launch
+# on the 160^3 drop impact (876 before part of the equilibrium's arithmetic
+# moved to the integer pipes).
+FP64_INSTR_PER_LIQUID_CELL_D3Q27_TRT = 434
 # DRAM bytes (read + write) per launch of the bulk kernel on the 256^3
 # workload, from one single-pass ncu capture of the autotuner's launches of
 # each variant, with the digest of the kernel sources the capture ran

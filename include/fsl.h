@@ -137,8 +137,12 @@ fsl_status fsl_init_fill(fsl_handle* h, const double* phi, const double* u0,
                          const unsigned char* obstacle, double h_ref);
 
 /* Advance nsteps time steps (asynchronous).  After an instability has been
- * latched, further steps do nothing.  Launch sequence is captured once into a
- * CUDA graph per distinct nsteps and replayed. */
+ * latched, further steps do nothing.  The launch sequence is captured once into
+ * a CUDA graph per distinct chunk of up to 64 steps and replayed.  A small
+ * domain (no bubble model, default variant) runs up to 512 steps in one
+ * cooperative launch when nsteps >= 4; the results are the same bits.  On the
+ * legacy default stream, or inside a capture of the caller's, the kernels of
+ * each step are launched one by one. */
 fsl_status fsl_step(fsl_handle* h, int nsteps);
 
 /* Observables (fsl_observe `what`).  host_out must hold `bytes` bytes. */
@@ -188,7 +192,8 @@ fsl_status fsl_destroy(fsl_handle* h);
  * FSL_ERR_ARG for an unknown lattice. */
 fsl_status fsl_lattice_table(int lattice, int* c3q, double* w);
 
-/* Number of kernel launches one fsl_step(1) issues. */
+/* Number of kernel launches one fsl_step(1) issues (without the sort of the
+ * interface list, one launch every eight steps). */
 int fsl_launches_per_step(const fsl_handle* h);
 
 /* Bulk stream-collide kernel of the FP32 / FP16 / BF16 storages (the FP64
