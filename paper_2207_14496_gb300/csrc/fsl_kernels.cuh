@@ -2954,6 +2954,11 @@ __device__ __forceinline__ void end_step_body(const Dev& d, const Geom& g) {
   }
   if (!ALONE || every > 0) {
     __threadfence();
+    // every warp of the block has read the step counter before its arrival is
+    // counted: the last block advances the counter, and a warp that read it
+    // late would take the next step for this one (trace it, or find it latched)
+    // and meet the block's barriers out of turn
+    __syncthreads();
     if (threadIdx.x == 0) last = atomicAdd(&ctrl->end_blocks, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!last) return;
