@@ -38,8 +38,11 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr long long kPlaneSkew = 512;  // elements added to every PDF plane
 
 enum Region {
-  R_PDF0, R_PDF1, R_FLAGS, R_CLAIM, R_PHI, R_PHINEW, R_MASS, R_RHO, R_KAPPA, R_MEX, R_LOST, R_PHIF,
-  R_LIF, R_LIF2, R_LFILL, R_LEMPTY, R_LNEW, R_LL2I, R_LRECV, R_LTILES, R_CTRL, R_TRACE, R_RED,
+  R_PDF0, R_PDF1, R_FLAGS, R_CLAIM, R_PHI, R_MASS, R_KAPPA, R_LOST, R_PHIF, R_LIF, R_LIF2,
+  // R_PHINEW .. R_LRECV: written and read within one step only, so that between
+  // steps their 44 bytes per cell, in one piece, are the scratch of fsl_observe
+  R_PHINEW, R_RHO, R_MEX, R_LFILL, R_LEMPTY, R_LNEW, R_LL2I, R_LRECV,
+  R_LTILES, R_CTRL, R_TRACE, R_RED,
   R_BLAB, R_BNEW, R_BK, R_BKNEW, R_BV, R_BVSEEN, R_BP, R_BHAS, R_SELF, R_COUNT
 };
 
@@ -140,7 +143,8 @@ void region_sizes(const fsl_config* c, const Geom& g, size_t* sz) {
       cells * sizeof(double);
   // the FP32 copy of the fill level that the 16/32-bit kernels read
   sz[R_PHIF] = c->precision == FSL_FP64 ? 0 : cells * sizeof(float);
-  for (int r = R_LIF; r <= R_LRECV; ++r) sz[r] = cells * sizeof(int);
+  for (int r : {R_LIF, R_LIF2, R_LFILL, R_LEMPTY, R_LNEW, R_LL2I, R_LRECV})
+    sz[r] = cells * sizeof(int);
   // tile lists of the shared-memory variants: up to one entry per 64 cells of a row
   sz[R_LTILES] = (size_t)((g.nx + 63) / 64) * g.ny * g.nz * sizeof(int);
   sz[R_CTRL] = sizeof(Ctrl);
@@ -606,11 +610,12 @@ fsl_status fsl_observe(fsl_handle* h, int what, void* host_out, size_t bytes) {
       if (bytes < (size_t)q * n * sizeof(double)) return FSL_ERR_ARG;
       double* o = static_cast<double*>(host_out);
       touch_pages(o, (size_t)q * n * sizeof(double));
-      // decoded into the other PDF buffer (the next step overwrites it), as many
-      // planes at a time as fit, and copied together
-      double* tmp = static_cast<double*>(h->d.pdf[cur ^ 1]);
-      const size_t room = (size_t)h->g.plane * q * storage_bytes(h->cfg.precision) / sizeof(double);
-      const int m = (int)std::min<size_t>(q, room / n);  // q / 4 planes or more
+      // decoded into the scratch of a step, as many planes at a time as fit,
+      // and copied together.  (The other PDF buffer is no scratch: the next step
+      // writes its fluid cells only, and the others are saved with the state.)
+      double* tmp = h->d.phinew;
+      const size_t room = (h->off[R_LTILES] - h->off[R_PHINEW]) / sizeof(double);
+      const int m = (int)std::min<size_t>(q, room / n);  // five planes or more
       for (int i = 0; i < q; i += m) {
         const int k = std::min(m, q - i);
         for (int j = 0; j < k; ++j)
