@@ -252,7 +252,10 @@ __device__ __forceinline__ double collide64(const double* fin, double* fout, con
   bool summed = false;
   if (FIXED) {
     // the density, left to right: near equilibrium f_0 (8/27 or 1/3 of rho) puts
-    // the partial sums in [1/4, 2); if they leave it, FP64 additions below
+    // the partial sums in [1/4, 2); if one leaves it, FP64 additions below.  The
+    // sums are tested before they are rounded: just below 1/4 the place that
+    // fix60_round drops to is too coarse, and 1/4 comes out.  (One that rounds up
+    // to 2 is right, and the next one is out of range unless it is below 2 again.)
     unsigned top = 0u;
     const Fix60 f0 = fix60_signed(fin[0], top);
     unsigned long long sum = f0.x;
@@ -260,8 +263,9 @@ __device__ __forceinline__ double collide64(const double* fin, double* fout, con
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
       const Fix60 f = fix60_signed(fin[i], top);
-      sum = fix60_round(sum + f.x, f.sticky);
+      sum += f.x;
       in = in && (sum >> 58) - 1u < 7u;
+      sum = fix60_round(sum, f.sticky);
     }
     summed = in && top < 0x3ff00000u;  // every |f_i| below 1
     rho = fix60_double(sum);
