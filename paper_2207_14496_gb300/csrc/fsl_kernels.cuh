@@ -36,6 +36,7 @@
 //   k_end_step        trace record, counters, step counter.
 #pragma once
 #include "fsl_lattice.cuh"
+#include "fsl_per_device.h"
 
 namespace fsl {
 
@@ -3258,6 +3259,33 @@ __global__ void k_export_plane(Dev d, Geom g, int cur, int i, double* dst) {
 }
 
 // ------------------------------------------------------------ launch table
+// Blocks of a kernel that are resident at once on the current device, at most
+// `most` per SM, after the kernel's opt-in to `smem` bytes of shared memory
+// there.  known: the kernel's own, kept by the caller.
+template <class Kernel>
+cudaError_t resident_blocks(PerDevice& known, Kernel* kernel, int threads, size_t smem, int most,
+                            int* blocks) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return known.get(
+      dev, blocks,
+      [&](int* n) {
+        int per_sm = 0, sms = 0;
+        cudaError_t f = cudaSuccess;
+        if (smem > 0)
+          f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (f == cudaSuccess)
+          f = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+        if (f == cudaSuccess) f = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (f == cudaSuccess && per_sm < 1) f = cudaErrorLaunchOutOfResources;
+        if (f == cudaSuccess) *n = (per_sm < most ? per_sm : most) * sms;
+        return f;
+      },
+      cudaSuccess);
+}
+constexpr int kAllResident = 1 << 20;
+
 template <int Q, class ST>
 struct Kernels {
   // the buffer parity is read on the device from the step counter, so the
@@ -3333,19 +3361,10 @@ struct Kernels {
   }
   template <int AX>
   static cudaError_t steps_as(const Dev& d, const Geom& g, const Phys& p, int n, cudaStream_t s) {
-    static int sms = 0;
-    if (sms == 0) {
-      cudaError_t e = cudaFuncSetAttribute(k_steps<Q, ST, AX>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIfSmem);
-      if (e != cudaSuccess) return e;
-      int per_sm = 0, dev = 0, k = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_steps<Q, ST, AX>, kStepsThreads, kIfSmem);
-      if (e == cudaSuccess) e = cudaGetDevice(&dev);
-      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&k, cudaDevAttrMultiProcessorCount, dev);
-      if (e != cudaSuccess) return e;
-      if (per_sm < 1) return cudaErrorLaunchOutOfResources;
-      sms = k;
-    }
+    static PerDevice known;
+    int sms = 0;
+    cudaError_t e = resident_blocks(known, k_steps<Q, ST, AX>, kStepsThreads, kIfSmem, 1, &sms);
+    if (e != cudaSuccess) return e;
     // a block per kStepsThreads cells, at most one per SM
     const long long want = (g.cells + kStepsThreads - 1) / kStepsThreads;
     cudaLaunchConfig_t cfg = {};
@@ -3358,7 +3377,7 @@ struct Kernels {
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_steps<Q, ST, AX>, d, g, p, n);
+    e = cudaLaunchKernelEx(&cfg, k_steps<Q, ST, AX>, d, g, p, n);
     // its barrier arrivals
     if (e == cudaSuccess) e = cudaMemsetAsync(&d.ctrl->bar, 0, sizeof(unsigned), s);
     return e;
@@ -3366,9 +3385,11 @@ struct Kernels {
   static constexpr size_t kIfSmem = Q == 19 ? sizeof(IfColumn<Q, typename ST::R>) : 0;
   template <int AX>
   static cudaError_t interface_pass_as(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
-    static const cudaError_t e =
-        cudaFuncSetAttribute(k_stream_collide_if<Q, ST, AX>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIfSmem);
+    // (the grid is kCellListBlocks, resident or not)
+    static PerDevice known;
+    int blocks = 0;
+    const cudaError_t e =
+        resident_blocks(known, k_stream_collide_if<Q, ST, AX>, 128, kIfSmem, kAllResident, &blocks);
     if (e != cudaSuccess) return e;
     k_stream_collide_if<Q, ST, AX><<<kCellListBlocks, 128, kIfSmem, s>>>(d, g, p);
     return cudaGetLastError();
@@ -3387,18 +3408,11 @@ struct Kernels {
   }
   // the conversion phase (k_convert), cooperative: one block per SM
   static cudaError_t convert(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
-    static int grid = 0;
-    if (grid == 0) {
-      int per_sm = 0, dev = 0, sms = 0;
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_convert<Q, ST>,
-                                                                    convert_threads<ST>(), 0);
-      if (e != cudaSuccess) return e;
-      e = cudaGetDevice(&dev);
-      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (e != cudaSuccess) return e;
-      if (per_sm < 1) return cudaErrorLaunchOutOfResources;
-      grid = sms;
-    }
+    static PerDevice known;
+    int grid = 0;
+    const cudaError_t e =
+        resident_blocks(known, k_convert<Q, ST>, convert_threads<ST>(), 0, 1, &grid);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -3481,20 +3495,12 @@ struct Kernels {
   template <int NS, int MINB, bool MULTI>
   static cudaError_t launch_tma_as(const Dev& d, const Geom& g, const Phys& p, const RowTiles& rt,
                                    cudaStream_t s) {
-    static int grid = 0;
+    static PerDevice known;
+    int grid = 0;
     constexpr size_t smem = BulkRing<Q, ST, NS>::bytes;
     auto* kernel = k_stream_collide_bulk<Q, ST, NS, MINB, MULTI>;
-    if (grid == 0) {
-      cudaError_t e =
-          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      int per_sm = 0, dev = 0, sms = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBulkThreads, smem);
-      if (e != cudaSuccess) return e;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      grid = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    const cudaError_t e = resident_blocks(known, kernel, kBulkThreads, smem, kAllResident, &grid);
+    if (e != cudaSuccess) return e;
     const int ntx = (g.nx + kBulkTX - 1) / kBulkTX;
     kernel<<<grid, kBulkThreads, smem, s>>>(d, g, p, ntx, rt);
     return cudaGetLastError();
@@ -3502,20 +3508,12 @@ struct Kernels {
   // persistent cp.async pipeline with S stages and at least MINB blocks per SM
   template <int S, int MINB>
   static cudaError_t launch_cpa(const Dev& d, const Geom& g, const Phys& p, cudaStream_t s) {
-    static int grid = 0;
+    static PerDevice known;
+    int grid = 0;
     constexpr size_t smem = CpRing<Q, ST, S>::bytes;
-    if (grid == 0) {
-      cudaError_t e = cudaFuncSetAttribute(k_stream_collide_cpa<Q, ST, S, MINB>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      int per_sm = 0, dev = 0, sms = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_cpa<Q, ST, S, MINB>,
-                                                        kCpThreads, smem);
-      if (e != cudaSuccess) return e;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      grid = (per_sm > 0 ? per_sm : 1) * sms;
-    }
+    const cudaError_t e = resident_blocks(known, k_stream_collide_cpa<Q, ST, S, MINB>, kCpThreads, smem,
+                                          kAllResident, &grid);
+    if (e != cudaSuccess) return e;
     const int ntx = (g.nx + kBulkTX - 1) / kBulkTX;
     k_stream_collide_cpa<Q, ST, S, MINB><<<grid, kCpThreads, smem, s>>>(d, g, p, ntx);
     return cudaGetLastError();
@@ -3560,18 +3558,12 @@ struct Kernels {
         if constexpr (half) return launch_tma<3, 4>(d, g, p, s);
       }
       if (v == 14 || v == 15) {
-        static int grid14 = 0, grid15 = 0;
-        int& grid = v == 14 ? grid14 : grid15;
-        if (grid == 0) {
-          int per_sm = 0, dev = 0, sms = 0;
-          cudaError_t e = v == 14
-              ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_c1<Q, ST, 8>, 128, 0)
-              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_c1<Q, ST, 6>, 128, 0);
-          if (e != cudaSuccess) return e;
-          cudaGetDevice(&dev);
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-          grid = (per_sm > 0 ? per_sm : 1) * sms;
-        }
+        static PerDevice known14, known15;
+        int grid = 0;
+        const cudaError_t e =
+            v == 14 ? resident_blocks(known14, k_stream_collide_c1<Q, ST, 8>, 128, 0, kAllResident, &grid)
+                    : resident_blocks(known15, k_stream_collide_c1<Q, ST, 6>, 128, 0, kAllResident, &grid);
+        if (e != cudaSuccess) return e;
         const int ntx = (g.nx + kWarpTX - 1) / kWarpTX;
         if (v == 14) k_stream_collide_c1<Q, ST, 8><<<grid, 128, 0, s>>>(d, g, p, ntx);
         else k_stream_collide_c1<Q, ST, 6><<<grid, 128, 0, s>>>(d, g, p, ntx);
@@ -3579,18 +3571,12 @@ struct Kernels {
       }
       if (v == 12 || v == 13) {
         // persistent warps over the 64-cell segment list: as many blocks as fit
-        static int grid12 = 0, grid13 = 0;
-        int& grid = v == 12 ? grid12 : grid13;
-        if (grid == 0) {
-          int per_sm = 0, dev = 0, sms = 0;
-          cudaError_t e = v == 12
-              ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_seg<Q, ST, 5>, 128, 0)
-              : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_seg<Q, ST, 4>, 128, 0);
-          if (e != cudaSuccess) return e;
-          cudaGetDevice(&dev);
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-          grid = (per_sm > 0 ? per_sm : 1) * sms;
-        }
+        static PerDevice known12, known13;
+        int grid = 0;
+        const cudaError_t e =
+            v == 12 ? resident_blocks(known12, k_stream_collide_seg<Q, ST, 5>, 128, 0, kAllResident, &grid)
+                    : resident_blocks(known13, k_stream_collide_seg<Q, ST, 4>, 128, 0, kAllResident, &grid);
+        if (e != cudaSuccess) return e;
         const int ntx = (g.nx + kWarpTX - 1) / kWarpTX;
         if (v == 12) k_stream_collide_seg<Q, ST, 5><<<grid, 128, 0, s>>>(d, g, p, ntx);
         else k_stream_collide_seg<Q, ST, 4><<<grid, 128, 0, s>>>(d, g, p, ntx);
@@ -3608,21 +3594,12 @@ struct Kernels {
         if constexpr (half) return launch_tma<4, 3>(d, g, p, s);
         else return launch_tma<3, 3>(d, g, p, s);
       } else if (v == 6) {
-        static int grid = 0;
+        static PerDevice known;
+        int grid = 0;
         constexpr size_t smem = WarpRing<Q, ST>::bytes;
-        if (grid == 0) {
-          cudaError_t e = cudaFuncSetAttribute(k_stream_collide_wtma<Q, ST>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
-          if (e != cudaSuccess) return e;
-          int per_sm = 0, dev = 0, sms = 0;
-          e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_wtma<Q, ST>,
-                                                            32 * kWarpsPerBlock, smem);
-          if (e != cudaSuccess) return e;
-          cudaGetDevice(&dev);
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-          grid = (per_sm > 0 ? per_sm : 1) * sms;
-        }
+        const cudaError_t e = resident_blocks(known, k_stream_collide_wtma<Q, ST>, 32 * kWarpsPerBlock,
+                                              smem, kAllResident, &grid);
+        if (e != cudaSuccess) return e;
         const int ntx = (g.nx + kWarpTX - 1) / kWarpTX;
         k_stream_collide_wtma<Q, ST><<<grid, 32 * kWarpsPerBlock, smem, s>>>(d, g, p, ntx);
       } else if (v == 7) {
