@@ -237,7 +237,11 @@ int fsl_launches_per_step(const fsl_handle* h);
  *   TMA_R96 (16-bit storages only): as TMA with three stages and four blocks
  *     per SM (at most 102 registers), sixteen consumer warps per SM.
  * DEFAULT picks by the domain: TMA from 2.5 million (padded) cells on and in
- * domains with obstacles, SEG_R128 from 200,000 cells on, PAIR_R128 below; the
+ * domains with obstacles, SEG_R128 from 200,000 cells on, PAIR_R128 below.
+ * With free-slip walls, beside which every variant pulls direction by
+ * direction, PAIR_R128; but SEG_R128 in D3Q19 from 200,000 cells on where at
+ * most 5 % of the cells lie beside a wall, and TMA in D3Q27 from 2.5 million
+ * cells on where at most 1 % do, x is periodic and there is no obstacle.  The
  * Python autotuner (paper_2207_14496_gb300.autotune) measures the variants
  * instead.
  * fsl_set_variant drops captured step graphs; FSL_ERR_ARG for an unknown

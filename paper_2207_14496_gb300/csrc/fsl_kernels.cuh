@@ -3456,6 +3456,25 @@ struct Kernels {
     k_export_plane<Q, ST><<<4 * 152, 256, 0, s>>>(d, g, cur, i, dst);
     return cudaGetLastError();
   }
+  // FSL_VARIANT_DEFAULT in domains with free-slip walls.  A liquid cell beside
+  // a wall or obstacle pulls direction by direction there (pull_near), a long
+  // chain of loads: walls across x end every row and tile with one, and a
+  // persistent kernel holds its other work up behind it.  Step times in us
+  // (pair_r128 / seg_r128 / tma):
+  //   D3Q27 drop impacts, walls all round: 128^3 FP16 164 / 189 / 235, 256^3 798 /
+  //   986 / 1188, FP32 828 / 1082 / 1715; free-slip walls across z only: 160^3 FP16
+  //   156 / 149 / 170, 200^3 253 / 221 / 213, 256^3 370 / 302 / 267
+  //   D3Q19 dam breaks: 150^3 FP16, walls all round 228 / 196 / 388, 300x300x100
+  //   427 / 327 / 556, walls across y only 302 / 228 / 232; 400x400x20, walls
+  //   across z 132 / 140 / 145
+  static int free_slip_variant(const Geom& g) {
+    // share of the cells that lie beside a wall
+    const double beside = (g.periodic[0] ? 0.0 : 2.0 / g.nx) + (g.periodic[1] ? 0.0 : 2.0 / g.ny) +
+                          (g.periodic[2] ? 0.0 : 2.0 / g.nz);
+    if (Q == 27 && g.periodic[0] && !g.has_obst && beside <= 0.01 && g.cells >= 2500000) return 4;
+    if (Q == 19 && beside <= 0.05 && g.cells >= 200000) return 13;
+    return 2;
+  }
   // resolved bulk-kernel variant of the 16/32-bit path
   static int variant_of(const Geom& g) {
     constexpr bool half = sizeof(typename ST::T) == 2;
@@ -3464,6 +3483,7 @@ struct Kernels {
       return g.variant;
     if ((g.variant == 5 || g.variant == 7 || g.variant == 11 || g.variant == 16) && half)
       return g.variant;
+    if (g.free_slip) return free_slip_variant(g);
     // FSL_VARIANT_DEFAULT, by measured step times (us, pair_r128 / seg_r128 /
     // tma; D3Q27 drop impacts n^3, D3Q19 dam breaks, tubes of obstacles):
     //   large domains fill the TMA ring of every SM: 200^3 FP16 332 / 314 / 243,
