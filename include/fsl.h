@@ -30,9 +30,9 @@
  *     fsl_workspace_bytes bytes, 256-byte aligned) and the CUDA stream.  The
  *     library never calls cudaMalloc/cudaFree; it mallocs only the small host
  *     handle and temporary host buffers inside fsl_observe.
- *   - Host threads: large host output buffers (fsl_observe, fsl_save) have their
- *     pages touched by a few short-lived threads before the copy; they have
- *     ended when the call returns.
+ *   - Host threads: large host output buffers (fsl_observe, fsl_save) whose
+ *     pages are not there yet have them touched by a few short-lived threads
+ *     before the copy; they have ended when the call returns.
  *   - Synchronisation: fsl_step is asynchronous on the bound stream.
  *     fsl_init_fill, fsl_observe, fsl_save and fsl_load synchronise the stream
  *     before returning, so host buffers may be reused immediately.
