@@ -359,6 +359,13 @@ fsl_status copy_field(fsl_handle* h, const void* dev, size_t elem, void* host) {
   return FSL_OK;
 }
 
+// Below so many cells the cell types and the bubble labels are copied as they
+// are and brought into their form on the host, above it by a kernel first
+// (types, us: 4,096 cells 24 on the host, 28 by the kernel; 65,536 cells 29 and
+// 29; 450,000 cells 54 and 32; labels: 1,024 cells 25 and 28, 4,096 28 and 28,
+// 65,536 94 and 30).
+const size_t kHostTypes = 65536, kHostLabels = 4096;
+
 const size_t kGraphChunk = 64;
 // Steps of a small domain per launch (k_steps): a few steps do not repay the
 // instruction fetch that a launch saves, and a launch should not hold the GPU
@@ -652,6 +659,13 @@ fsl_status fsl_observe(fsl_handle* h, int what, void* host_out, size_t bytes) {
     }
     case FSL_OBS_FIELD_TYPES: {
       if (bytes < n) return FSL_ERR_ARG;
+      if (n < kHostTypes) {
+        st = copy_field(h, h->d.flags, 1, host_out);
+        if (st != FSL_OK) return st;
+        unsigned char* o = static_cast<unsigned char*>(host_out);
+        for (size_t k = 0; k < n; ++k) o[k] &= F_TYPE;
+        return FSL_OK;
+      }
       touch_pages(host_out, n);
       uint8_t* tmp = reinterpret_cast<uint8_t*>(h->d.phinew);  // scratch between steps
       k_export_types<<<4 * 152, 256, 0, h->stream>>>(h->d, h->g, tmp);
@@ -674,6 +688,14 @@ fsl_status fsl_observe(fsl_handle* h, int what, void* host_out, size_t bytes) {
       int* o = static_cast<int*>(host_out);
       if (!h->g.bubbles) {
         for (size_t k = 0; k < n; ++k) o[k] = -1;
+        return FSL_OK;
+      }
+      if (n < kHostLabels) {
+        st = copy_field(h, h->d.blab, sizeof(int), host_out);
+        if (st != FSL_OK) return st;
+        // padded cell index -> dense index x + nx (y + ny z)
+        for (size_t k = 0; k < n; ++k)
+          if (o[k] >= 0) o[k] = (o[k] % h->g.sx) + h->g.nx * (o[k] / h->g.sx);
         return FSL_OK;
       }
       touch_pages(host_out, n * sizeof(int));
