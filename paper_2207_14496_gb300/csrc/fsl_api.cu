@@ -649,8 +649,7 @@ fsl_status fsl_observe(fsl_handle* h, int what, void* host_out, size_t bytes) {
       const int m = (int)std::min<size_t>(q, room / n);  // five planes or more
       for (int i = 0; i < q; i += m) {
         const int k = std::min(m, q - i);
-        for (int j = 0; j < k; ++j)
-          FSL_CK(h->L->export_pdf(h->d, h->g, h->p, cur, i + j, tmp + (size_t)j * n, h->stream));
+        FSL_CK(h->L->export_pdf(h->d, h->g, h->p, cur, i, k, tmp, h->stream));
         FSL_CK(cudaMemcpyAsync(o + (size_t)i * n, tmp, (size_t)k * n * sizeof(double),
                                cudaMemcpyDeviceToHost, h->stream));
       }

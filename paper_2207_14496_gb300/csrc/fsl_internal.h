@@ -174,8 +174,8 @@ struct Launch {
   // max |u| over fluid cells into out (device double)
   cudaError_t (*max_velocity)(const Dev&, const Geom&, const Phys&, int cur, double* out,
                               cudaStream_t);
-  // decode plane i of pdf[cur] into dst (device, nx*ny*nz doubles, unpadded)
-  cudaError_t (*export_pdf)(const Dev&, const Geom&, const Phys&, int cur, int i, double* dst,
+  // decode planes i .. i + k - 1 of pdf[cur] into dst (device, k*nx*ny*nz doubles, unpadded)
+  cudaError_t (*export_pdf)(const Dev&, const Geom&, const Phys&, int cur, int i, int k, double* dst,
                             cudaStream_t);
   // work lists the bulk kernel needs (interface cells, liquid tiles), or null
   cudaError_t (*pre_bulk)(const Dev&, const Geom&, const Phys&, cudaStream_t);
