@@ -209,8 +209,9 @@ int fsl_launches_per_step(const fsl_handle* h);
  *     five and six blocks per SM); PAIR_R128 collides them one after the
  *     other (128 registers);
  *   TMA: persistent, tiles of 256 cells with liquid (listed by a pre-pass; of
- *     several whole rows where a row has at most 128 cells) staged in shared memory by bulk copies through a ring of
- *     mbarrier-guarded stages, one producer warp and four consumer warps;
+ *     several whole rows where a row has at most 128 cells) staged in shared
+ *     memory by bulk copies through a ring of mbarrier-guarded stages, one
+ *     producer warp and four consumer warps;
  *   QUAD_64 (16-bit storages only): four cells per thread, 64 threads per
  *     block, one 8-byte load per direction kept packed until the collision;
  *   WARP_TMA: persistent, every warp streams its own 64-cell row segments

@@ -13,6 +13,11 @@ the variant needs) and keeps the fastest; `tune_batch` tunes one
 representative per distinct (lattice, storage, shape) and applies the pick
 to every simulation of that kind.  Picks can be kept in a JSON file so that a
 later run skips the measurements.
+
+What is compared is the variants named.  A small domain left at "default"
+(FSL_VARIANT_DEFAULT) runs many steps in one launch (include/fsl.h, fsl_step)
+and steps faster than with any of them, so there is nothing to tune there;
+`tune_step` takes "default" as a candidate.
 """
 from __future__ import annotations
 

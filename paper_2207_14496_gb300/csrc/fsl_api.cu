@@ -368,8 +368,11 @@ const size_t kHostTypes = 65536, kHostLabels = 4096;
 
 const size_t kGraphChunk = 64;
 // Steps of a small domain per launch (k_steps): a few steps do not repay the
-// instruction fetch that a launch saves, and a launch should not hold the GPU
-// for more than some ten milliseconds.
+// instruction fetch that a launch saves, and a launch does not end before its
+// steps do: 512 of them hold their SMs for 14 ms (64x64 FP32) to 35 ms (64x64
+// FP64).  Handles on streams of their own gain by it all the same: 512 steps of
+// 16 waves of 64x64 cells, ms, one launch per kernel / k_steps: FP32 309 / 23,
+// FP64 318 / 47; eight of 150x150, FP64: 201 / 98.
 const int kStepsMin = 4, kStepsMost = 512;
 // The interface list is put back into memory order (k_sort_interface) every so
 // many steps: inside the captured graphs of that many steps or more, before
